@@ -522,72 +522,54 @@ __global__ void __launch_bounds__(PAR ? BFS_THREADS_PAR : BFS_THREADS, PAR ? 2 :
             break;
         }
     }
-    if (tid == 0 && blockIdx.x == 0) A.sync[7] = (uint32_t)L;
-    // work counters (one atomic per warp and counter)
+    // work counters of the batch (sb_stats), one atomic per warp and counter
+    unsigned long long* acc = (unsigned long long*)(A.sync + 16);
+    if (tid == 0 && blockIdx.x == 0) {
+        atomicMax(acc, (unsigned long long)L);
+        atomicAdd(acc + 1, 1ull);
+    }
     for (int d = 16; d; d >>= 1) {
         n_scan += __shfl_xor_sync(0xffffffffu, n_scan, d);
         n_hash += __shfl_xor_sync(0xffffffffu, n_hash, d);
         n_hash_hub += __shfl_xor_sync(0xffffffffu, n_hash_hub, d);
     }
     if ((tid & 31) == 0) {
-        atomicAdd((unsigned long long*)(A.sync + 8), (unsigned long long)n_scan);
-        atomicAdd((unsigned long long*)(A.sync + 10), (unsigned long long)n_hash);
-        atomicAdd((unsigned long long*)(A.sync + 14), (unsigned long long)n_hash_hub);
+        atomicAdd(acc + 2, (unsigned long long)n_scan);
+        atomicAdd(acc + 3, (unsigned long long)n_hash);
+        atomicAdd(acc + 5, (unsigned long long)n_hash_hub);
     }
 }
 
 // ------------------------------------------------------------ BFS set-up
-__global__ void k_bfs_init(int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_t* vis, uint64_t* fr0, uint64_t* fr1,
-                           uint64_t* lab, int32_t* done)
+// State of one BFS launch before its roots: visited bits, the level-1
+// frontier, labels, split-row keys, level counters and barrier words.  (The
+// other frontier buffer is written for every vertex at level 2, before its
+// first read.  The error word sync[6] is cleared per batch, so that an error
+// of an earlier launch stays.)
+__global__ void k_bfs_init(int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_t* vis, uint64_t* fr1, uint64_t* lab,
+                           int32_t* done, int64_t nh, uint64_t* hubnew, uint64_t* hubbest, uint32_t* sync)
 {
-    int64_t total = n * Wb;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (i0 < 6) sync[i0] = 0;
+    const int64_t total = n * Wb;
+    for (int64_t i = i0; i < total; i += step) {
         int64_t v = i / Wb;
         int w = (int)(i - v * Wb);
         int64_t trees = K - 64 * (int64_t)(w0 + w);  // trees of this word
         uint64_t active = trees >= 64 ? ~0ull : ((1ull << trees) - 1ull);
         vis[i] = ~active;
-        fr0[i] = 0;
         fr1[i] = 0;
         lab[v * Wt + w0 + w] = 0;
         if (w == 0) done[v] = -1;
     }
-}
-
-__global__ void k_hub_init(int64_t nh, int Wb, uint64_t* hubnew, uint64_t* hubbest)
-{
-    int64_t total = nh * Wb * 64;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = i0; i < nh * Wb * 64; i += step) {
         hubbest[i] = ~0ull;
         if (i < nh * Wb) hubnew[i] = 0;
     }
 }
 
-// root of every tree of this launch in every graph (one graph unless voff)
-__global__ void k_bfs_roots(int64_t n, int Wb, int w0, int64_t K, uint64_t S, const int64_t* tree0p, uint64_t* vis,
-                            uint64_t* fr0, int32_t* parents, const int32_t* voff, int64_t G)
-{
-    const int64_t tree0 = *tree0p;
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t per = 64 * (int64_t)Wb;
-    if (x >= per * G) return;
-    const int64_t g = x / per;
-    const int64_t i = x - g * per;      // tree within this launch
-    const int64_t tb = 64 * (int64_t)w0 + i;  // tree within the batch
-    if (tb >= K) return;
-    const uint64_t key = sb_tree_key(S, tree0 + tb);
-    const int64_t base = voff ? voff[g] : 0;
-    const int64_t ng = voff ? voff[g + 1] - voff[g] : n;
-    const uint32_t r = (uint32_t)(base + sb_root(key, ng));
-    int w = (int)(i >> 6);
-    unsigned long long bit = 1ull << (i & 63);
-    atomicOr((unsigned long long*)(vis + (int64_t)r * Wb + w), bit);
-    atomicOr((unsigned long long*)(fr0 + (int64_t)r * Wb + w), bit);
-    if (parents) parents[tb * n + r] = -1;
-}
-
-// BFS level 1, top-down: a neighbour v of tree t's root r joins the tree at
-// level 1 with r as its parent (the only vertex of level 0, so no hash
+// Roots and BFS level 1, top-down: a neighbour v of tree t's root r joins the
+// tree at level 1 with r as its parent (the only vertex of level 0, so no hash
 // decides), label lab(r) ^ neg(r, v) = neg(r, v).  One warp per (graph,
 // tree of the launch); trees of one word may reach the same vertex, hence
 // the atomics.  Frontier of level 1 -> fr1 (read as the current frontier of
@@ -610,6 +592,10 @@ __global__ void k_bfs_level1(int64_t n, int Wb, int Wt, int w0, int64_t K, uint6
     const int64_t r = base + sb_root(key, ng);
     const int w = (int)(i >> 6);
     const unsigned long long bit = 1ull << (i & 63);
+    if (lane == 0) {
+        atomicOr((unsigned long long*)(vis + r * Wb + w), bit);
+        if (parents) parents[tb * n + r] = -1;
+    }
     for (int32_t j = rowptr[r] + lane; j < rowptr[r + 1]; j += 32) {
         const uint32_t cv = (uint32_t)col[j];
         const int64_t v = cv & SB_ID_MASK;
@@ -620,10 +606,15 @@ __global__ void k_bfs_level1(int64_t n, int Wb, int Wt, int w0, int64_t K, uint6
     }
 }
 
-// canonical flip per graph and word: the raw label of the graph's vertex 0
-__global__ void k_flip(const uint64_t* lab, int W, uint64_t* flipw, const int32_t* voff, int64_t G)
+// canonical flip per graph and word (the raw label of the graph's vertex 0),
+// and the state-hash sums cleared for k_state_hash_tab; one thread per hash
+__global__ void k_flip(const uint64_t* lab, int W, uint64_t* flipw, const int32_t* voff, int64_t G,
+                       unsigned long long* H, unsigned long long* wsum)
 {
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= 64 * (int64_t)W * G) return;
+    H[x] = 0;
+    if (x < G) wsum[x] = 0;
     if (x >= (int64_t)W * G) return;
     const int64_t g = x / W;
     const int w = (int)(x - g * W);
@@ -646,6 +637,11 @@ __global__ void k_flip(const uint64_t* lab, int W, uint64_t* flipw, const int32_
 #define HT_THREADS 256
 #define HT_WARPS (HT_THREADS / 32)
 #define HT_WPW 8  // words per warp: 64 words over 8 warps
+// Fewest groups a block takes.  Groups of one block run one after the other,
+// so a small graph wants many blocks; each block ends with one atomic per tree.
+// 2 instead of 16: 25.9 -> 4.9 us at n = 1000, 64 trees, 50 -> 27 us at
+// n = 95,000, 1000 trees; from 39,000 vertices on the grid is full either way.
+#define HT_MIN_GROUPS 2
 
 __global__ void __launch_bounds__(HT_THREADS, 4) k_state_hash_tab(const uint64_t* __restrict__ lab, int64_t n, int W,
                                                                   const uint64_t* __restrict__ weight,
@@ -757,17 +753,6 @@ __global__ void k_canon_out(const uint64_t* __restrict__ lab, int64_t total, int
     }
 }
 
-__global__ void k_fold_stats(const uint32_t* sync, unsigned long long* acc)
-{
-    const unsigned long long L = sync[7];
-    if (L > acc[0]) acc[0] = L;
-    acc[1] += 1;
-    acc[2] += *(const unsigned long long*)(sync + 8);
-    acc[3] += *(const unsigned long long*)(sync + 10);
-    acc[4] += *(const unsigned long long*)(sync + 12);
-    acc[5] += *(const unsigned long long*)(sync + 14);
-}
-
 // --------------------------------------------------------------- host side
 static int group_for(int Wb)
 {
@@ -825,25 +810,16 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
     }
     const size_t smem = smem_for(qcap);
     if (per_sm < 1) return sb_fail(c, SB_ERR_CUDA, "BFS kernel does not fit on an SM");
-    unsigned nblocks = (unsigned)(per_sm * c->num_sms);
+    // one group per work item at most: every further block would only lengthen
+    // the grid barriers (1000 vertices, one word: 8 blocks instead of 760)
+    unsigned nblocks = (unsigned)std::max<int64_t>(
+        1, std::min<int64_t>((int64_t)per_sm * c->num_sms, sb_cdiv(c->n_items, BD / G)));
     const int64_t n = c->n;
-    unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(n * Wb, 256), (int64_t)c->num_sms * 16);
-    k_bfs_init<<<g, 256, 0, c->stream>>>(n, Wb, c->W, w0, c->K, c->vis, c->fr0, c->fr1, c->labels, c->done);
-    SB_TRY(sb_after_launch(c, "k_bfs_init"));
-    if (c->n_hubs > 0) {
-        unsigned gh = (unsigned)std::min<int64_t>(sb_cdiv(c->n_hubs * Wb * 64, 256), (int64_t)c->num_sms * 16);
-        k_hub_init<<<gh, 256, 0, c->stream>>>(c->n_hubs, Wb, c->hubnew, c->hubbest);
-        SB_TRY(sb_after_launch(c, "k_hub_init"));
-    }
     const int64_t ngraphs = c->batch_G > 0 ? c->batch_G : 1;
-    k_bfs_roots<<<(unsigned)sb_cdiv(64 * Wb * ngraphs, 256), 256, 0, c->stream>>>(
-        n, Wb, w0, c->K, sb_seed_key(c->seed), sb_tree0_ptr(c->sync), c->vis, c->fr0, parents,
-        c->batch_G > 0 ? c->b_voff : nullptr, ngraphs);
-    SB_TRY(sb_after_launch(c, "k_bfs_roots"));
-    // level counters and barrier words of this launch (the error word sync[6]
-    // is cleared per batch, so that an error of an earlier launch stays)
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->sync, 0, sizeof(uint32_t) * 6, c->stream));
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->sync + 7, 0, sizeof(uint32_t) * 9, c->stream));
+    unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(std::max(n, c->n_hubs * 64) * Wb, 256), (int64_t)c->num_sms * 16);
+    k_bfs_init<<<g, 256, 0, c->stream>>>(n, Wb, c->W, w0, c->K, c->vis, c->fr1, c->labels, c->done, c->n_hubs,
+                                         c->hubnew, c->hubbest, c->sync);
+    SB_TRY(sb_after_launch(c, "k_bfs_init"));
     {
         const int64_t warps = 64 * (int64_t)Wb * ngraphs;
         k_bfs_level1<<<(unsigned)sb_cdiv(warps * 32, 256), 256, 0, c->stream>>>(
@@ -893,18 +869,21 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
         cfg.numAttrs = 1;
         SbProf prof(c, SB_PROF_BFS);
         SB_CHECK_CUDA(c, cudaLaunchKernelExC(&cfg, fn, args));
-        SB_TRY(sb_after_launch(c, "k_bfs"));
+        return sb_after_launch(c, "k_bfs");
     }
-    k_fold_stats<<<1, 1, 0, c->stream>>>(c->sync, (unsigned long long*)(c->sync + 16));
-    return sb_after_launch(c, "k_fold_stats");
 }
 
-// *p = v, or *p += add when add != 0 (the device copy of the first tree)
-__global__ void k_set_i64(int64_t* p, int64_t v, int64_t add)
+// Start of a batch: work counters, error word and the device copy of the
+// first tree.
+__global__ void k_batch_begin(uint32_t* sync, int64_t tree0)
 {
-    if (add) *p += add;
-    else *p = v;
+    if (threadIdx.x < 16) sync[16 + threadIdx.x] = 0;
+    if (threadIdx.x == 16) sync[6] = 0;
+    if (threadIdx.x == 17) *sb_tree0_ptr(sync) = tree0;
 }
+
+// moves the device copy of the first tree on
+__global__ void k_add_i64(int64_t* p, int64_t add) { *p += add; }
 
 // errors of one step kept across the steps of sb_batch_steps: BFS barrier
 // (sync[6]) and scorer tile copies (sync[28]) into sync[34]
@@ -929,14 +908,18 @@ __global__ void k_fill_i32(int32_t* p, int64_t n, int32_t v)
         p[i] = v;
 }
 
-static sb_status check_sync_error(sb_ctx* c)
+// Waits for the stream and reports the sampler's error word, and the scorer's
+// when it has just been enqueued (one copy covers both).
+static sb_status check_sync_error(sb_ctx* c, bool scored = false)
 {
-    uint32_t err = 0;
-    SB_CHECK_CUDA(c, cudaMemcpyAsync(&err, c->sync + 6, sizeof(err), cudaMemcpyDeviceToHost, c->stream));
+    uint32_t w[23] = {0};  // sync[6 .. 28]
+    SB_CHECK_CUDA(c, cudaMemcpyAsync(w, c->sync + 6, sizeof(w), cudaMemcpyDeviceToHost, c->stream));
     SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
+    const uint32_t err = w[0];
     if (err & 1u) return sb_fail(c, SB_ERR_TIMEOUT, "BFS grid barrier timed out");
     if (err & 2u) return sb_fail(c, SB_ERR_DEVICE_CHECK, "BFS exceeded n levels");
     if (err & 4u) return sb_fail(c, SB_ERR_DEVICE_CHECK, "Kruskal trees did not span their graph");
+    if (scored && w[22]) return sb_fail(c, SB_ERR_TIMEOUT, "scorer tile copy timed out");
     return SB_OK;
 }
 
@@ -965,26 +948,23 @@ sb_status sb_batch_begin(sb_ctx* c, uint64_t seed, int64_t tree_begin, int64_t K
     c->W = W;
     c->counts_valid = false;
     c->batch_in_cloud = false;
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->sync + 16, 0, sizeof(uint32_t) * 16, c->stream));
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->sync + 6, 0, sizeof(uint32_t), c->stream));
-    k_set_i64<<<1, 1, 0, c->stream>>>(sb_tree0_ptr(c->sync), tree_begin, 0);
-    return sb_after_launch(c, "k_set_i64");
+    k_batch_begin<<<1, 32, 0, c->stream>>>(c->sync, tree_begin);
+    return sb_after_launch(c, "k_batch_begin");
 }
 
 sb_status sb_batch_end(sb_ctx* c)
 {
     const int64_t n = c->n, G = c->batch_G > 0 ? c->batch_G : 1;
     const int W = c->W;
-    k_flip<<<(unsigned)sb_cdiv((int64_t)W * G, 256), 256, 0, c->stream>>>(c->labels, W, c->flipw,
-                                                                          c->batch_G > 0 ? c->b_voff : nullptr, G);
-    SB_TRY(sb_after_launch(c, "k_flip"));
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->hashes, 0, sizeof(uint64_t) * 64 * W * G, c->stream));
     SB_TRY(sb_ensure(c, (void**)&c->hwsum, &c->hwsum_cap, sizeof(uint64_t) * (size_t)G));
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->hwsum, 0, sizeof(uint64_t) * (size_t)G, c->stream));
+    k_flip<<<(unsigned)sb_cdiv(64 * (int64_t)W * G, 256), 256, 0, c->stream>>>(
+        c->labels, W, c->flipw, c->batch_G > 0 ? c->b_voff : nullptr, G, (unsigned long long*)c->hashes,
+        (unsigned long long*)c->hwsum);
+    SB_TRY(sb_after_launch(c, "k_flip"));
     {
         SbProf prof(c, SB_PROF_HASH);
         const int64_t ngroups = sb_cdiv(n, 32);
-        const int64_t nblk = std::max<int64_t>(1, std::min<int64_t>((int64_t)c->num_sms * 4, sb_cdiv(ngroups, 16)));
+        const int64_t nblk = std::max<int64_t>(1, std::min<int64_t>((int64_t)c->num_sms * 4, sb_cdiv(ngroups, HT_MIN_GROUPS)));
         const int64_t per = sb_cdiv(ngroups, nblk);
         k_state_hash_tab<<<(unsigned)sb_cdiv(ngroups, per), HT_THREADS, 0, c->stream>>>(
             c->labels, n, W, c->vweight, c->batch_G > 0 ? c->vgid : nullptr, 64 * (int64_t)W, per,
@@ -1074,8 +1054,8 @@ static sb_status batch_step_enqueue(sb_ctx* c)
     SB_TRY(sb_batch_cloud_enqueue(c, c->bs_ns, c->bs_fm));
     k_fold_min<<<(unsigned)sb_cdiv(G, 256), 256, 0, c->stream>>>(c->bs_frmin, c->bs_fm, G);
     SB_TRY(sb_after_launch(c, "k_fold_min"));
-    k_set_i64<<<1, 1, 0, c->stream>>>(sb_tree0_ptr(c->sync), 0, c->K);
-    return sb_after_launch(c, "k_set_i64");
+    k_add_i64<<<1, 1, 0, c->stream>>>(sb_tree0_ptr(c->sync), c->K);
+    return sb_after_launch(c, "k_add_i64");
 }
 
 // Captures one step into a CUDA graph (or reuses the captured one while its
@@ -1182,8 +1162,10 @@ extern "C" sb_status sb_frustration(sb_ctx* c, int32_t* counts_out, uint64_t* ha
     if (!c) return SB_ERR_ARG;
     if (!c->has_batch) return sb_fail(c, SB_ERR_STATE, "no sampled batch");
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
-    SB_TRY(check_sync_error(c));
-    SB_TRY(sb_score_batch(c));
+    const bool score = !c->counts_valid;
+    if (score) SB_TRY(sb_score_enqueue(c));  // behind the sampler; one wait then covers both
+    SB_TRY(check_sync_error(c, score && c->m > 0));
+    c->counts_valid = true;
     if (c->batch_G > 0) {
         // per graph: K entries, packed graph after graph
         const size_t KP = 64 * (size_t)c->W, K = (size_t)c->K, G = (size_t)c->batch_G;

@@ -104,11 +104,15 @@ __device__ __forceinline__ uint32_t gl_emit(const GlArgs& A, int64_t v, int64_t 
 // of SL*VEC columns).  The segments run one after the other over the whole
 // grid, so one segment's columns of G (n x SL*VEC floats; 84 MB for 656k
 // vertices at 32 columns) stay in L2 while every row gathers from them.
-// Within a segment the sub-warps take blocks of GL_ITEM_BLOCK consecutive
-// items in turn: the chunks of one long row spread over many sub-warps, and a
-// block (rows in vertex order) rarely crosses a graph of a batch.
+// Within a segment the sub-warps take blocks of IB consecutive items in turn:
+// the chunks of one long row spread over many sub-warps, and a block (rows in
+// vertex order) rarely crosses a graph of a batch.  A graph too small for
+// every sub-warp to get GL_ROWS_PER_SUB rows takes them one at a time: with
+// blocks of 16, 1000 rows kept 63 of 4864 warps busy, each with 16 rows in
+// turn (33.7 us a descent step at 5 columns, now 6.4).
 #define GL_ITEM_BLOCK 16
-template <int VEC, int SL, bool STEP>
+#define GL_ROWS_PER_SUB 32
+template <int VEC, int SL, bool STEP, int IB>
 __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlArgs A)
 {
     extern __shared__ uint32_t gsm[];
@@ -132,15 +136,15 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
     // split-row chunks one at a time, then whole rows by blocks: work unit w
     // covers items [lo(w), hi(w))
     const int64_t nsplit = A.n_split_items;
-    const int64_t nunits = nsplit + sb_cdiv(A.n_items - nsplit, GL_ITEM_BLOCK);
+    const int64_t nunits = nsplit + sb_cdiv(A.n_items - nsplit, IB);
     const bool wantF = STEP && A.F != nullptr;
     for (int seg = 0; seg < nseg; seg++) {
         const int r0 = seg * seg_w + sl * VEC;
         const bool act = r0 < R;
         GlCols<VEC> cols;
         for (int64_t wu = sub_id; wu < nunits; wu += subs_total)
-        for (int64_t it = wu < nsplit ? wu : nsplit + (wu - nsplit) * GL_ITEM_BLOCK,
-                     it_end = wu < nsplit ? wu + 1 : min(A.n_items, nsplit + (wu - nsplit + 1) * GL_ITEM_BLOCK);
+        for (int64_t it = wu < nsplit ? wu : nsplit + (wu - nsplit) * IB,
+                     it_end = wu < nsplit ? wu + 1 : min(A.n_items, nsplit + (wu - nsplit + 1) * IB);
              it < it_end; it++) {
             const sb_bfs_item itm = A.items[it];
             const int64_t g = A.vgid ? A.vgid[itm.v] : 0;
@@ -466,20 +470,32 @@ static GlArgs gl_args(sb_ctx* c, int R)
     return A;
 }
 
+template <bool STEP, int IB>
+static const void* gl_rows_kernel(bool vec4, int64_t lanes)
+{
+    return !vec4        ? (const void*)k_gl_rows<1, 32, STEP, IB>
+           : lanes == 32 ? (const void*)k_gl_rows<4, 32, STEP, IB>
+           : lanes == 16 ? (const void*)k_gl_rows<4, 16, STEP, IB>
+                         : (const void*)k_gl_rows<4, 8, STEP, IB>;
+}
+
 template <bool STEP>
 static sb_status gl_rows_launch(sb_ctx* c, GlArgs& A)
 {
     const bool vec4 = (A.R % 4 == 0) && (((uintptr_t)A.gin & 15) == 0);
     const int64_t lanes = c->tune[SB_TUNE_GL_LANES];
-    const void* fn = !vec4        ? (const void*)k_gl_rows<1, 32, STEP>
-                     : lanes == 32 ? (const void*)k_gl_rows<4, 32, STEP>
-                     : lanes == 16 ? (const void*)k_gl_rows<4, 16, STEP>
-                                   : (const void*)k_gl_rows<4, 8, STEP>;
+    const int subs = GL_THREADS / (vec4 && lanes != 32 ? (lanes == 16 ? 16 : 8) : 32);
+    const int64_t rows = A.n_items - A.n_split_items;
+    const bool small = rows < (int64_t)c->num_sms * GL_ROWS_MIN_BLOCKS * subs * GL_ROWS_PER_SUB;
+    const void* fn = small ? gl_rows_kernel<STEP, 1>(vec4, lanes) : gl_rows_kernel<STEP, GL_ITEM_BLOCK>(vec4, lanes);
     size_t smem = STEP ? sizeof(uint32_t) * 2 * (size_t)A.R : 0;
     if (smem > 48 * 1024) SB_CHECK_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     SB_CHECK_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, GL_THREADS, smem));
-    unsigned blocks = (unsigned)(c->num_sms * std::max(per_sm, 1));
+    // blocks without a work unit are not launched
+    const int64_t units = A.n_split_items + sb_cdiv(rows, small ? 1 : GL_ITEM_BLOCK);
+    unsigned blocks = (unsigned)std::max<int64_t>(
+        1, std::min<int64_t>((int64_t)c->num_sms * std::max(per_sm, 1), sb_cdiv(units, subs)));
     void* args[] = {&A};
     SbProf prof(c, SB_PROF_GL_ROWS);
     SB_CHECK_CUDA(c, cudaLaunchKernel(fn, dim3(blocks), dim3(GL_THREADS), args, smem, c->stream));

@@ -142,6 +142,7 @@ struct sb_ctx {
     uint64_t* hubnew = nullptr;
     uint64_t* hubbest = nullptr;
     uint32_t* sync = nullptr;     // [0..2] level counters, [4] barrier count, [5] barrier gen, [6] error,
+                                  // [16..27] work counters of the batch (sb_stats), [28] scorer error,
                                   // [32..33] first tree of the batch (int64, read by the kernels),
                                   // [34] sticky errors of sb_batch_steps
     size_t bfs_cap_words = 0;
