@@ -279,8 +279,9 @@ sb_status sb_sample_trees(sb_ctx* ctx, uint64_t seed, int64_t tree_begin, int64_
  * a pure function of (seed, t).  Works on a single graph and on a batch.
  * K >= 1 (at most 64 * 64 per call).  in_tree_out (device, K x m bytes,
  * nullable; edge order of sb_graph_edges): 1 where the edge is in the tree.
- * Scratch: 36 bytes per (vertex, tree); a pass of trees takes at most
- * 16 GiB and half the free device memory (at least 64 trees per pass).  The
+ * Scratch: 17 bytes per (vertex, tree), plus 4 per tree and 32 CSR entries
+ * where light edges are searched first; a pass of trees takes at most
+ * 32 GiB and half the free device memory (at least 64 trees per pass).  The
  * context keeps it for the next call until a graph is loaded or the context
  * is destroyed.
  * Errors: SB_ERR_ARG, SB_ERR_STATE (no graph), SB_ERR_OOM; a tree that does

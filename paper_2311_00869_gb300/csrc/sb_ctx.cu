@@ -202,12 +202,12 @@ void sb_release_batch(sb_ctx* c)
     SB_FREE(hubbest);
     SB_FREE(mst_P);
     SB_FREE(mst_R);
-    SB_FREE(mst_Y);
-    SB_FREE(mst_L);
     SB_FREE(mst_B);
-    SB_FREE(mst_win);
+    SB_FREE(mst_done);
+    SB_FREE(mst_big);
+    SB_FREE(mst_light);
     SB_FREE(mst_flags);
-    c->mst_cap = 0;
+    c->mst_cap = c->mst_done_cap = c->mst_big_cap = c->mst_light_cap = 0;
     c->labels_cap = 0;
     c->bfs_cap_words = 0;
     c->has_batch = false;

@@ -150,11 +150,14 @@ struct sb_ctx {
     // Kruskal (Boruvka) scratch, [vertex][tree of the pass]
     uint32_t* mst_P = nullptr;    // parent << 1 | parity to it
     uint32_t* mst_R = nullptr;    // root << 1 | parity to it, at the start of a round
-    uint32_t* mst_Y = nullptr;    // lightest outgoing neighbour | neg << 31, or SB_MST_DEAD
-    uint64_t* mst_L = nullptr;    // its weight
     uint64_t* mst_B = nullptr;    // lightest outgoing weight of the component this vertex roots
-    int2* mst_win = nullptr;      // (inside endpoint, outside endpoint | neg << 31) of that edge, or -1
-    int32_t* mst_flags = nullptr; // [r] = 1 when round r - 1 merged something
+    uint32_t* mst_done = nullptr; // [work item][32 trees]: nothing left to find
+    size_t mst_done_cap = 0;
+    uint32_t* mst_big = nullptr;  // [graph][tree]: root of the component that does not search
+    size_t mst_big_cap = 0;
+    uint32_t* mst_light = nullptr; // [32 entries of a row][tree]: bit per light entry
+    size_t mst_light_cap = 0;
+    int32_t* mst_flags = nullptr; // mode of every round, then 1 for rounds that merged something
     size_t mst_cap = 0;           // (vertex, tree) slots held
 
     // cloud

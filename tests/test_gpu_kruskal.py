@@ -156,3 +156,35 @@ def test_kruskal_argument_and_state_errors(P):
         _check(P, sb, g, seed=1, t0=0, K=4096)
     finally:
         sb.close()
+
+
+@pytest.mark.parametrize("n,m,hub", [(1001, 106000, 0), (3000, 105000, 2500), (11000, 105100, 0)])
+def test_kruskal_light_rounds_match_oracle(P, n, m, hub):
+    """Graphs large and dense enough for rounds over light edges only (2^26
+    pairs of an edge's end and a tree, 9 edges per vertex), with rows of up to
+    2500 entries (several chunks), alone and as graphs of one batch with a
+    sparse one."""
+    K = 300
+    n, u, v, s = synth.er_graph(n, m, 0.3, seed=n)
+    if hub:
+        u = np.concatenate([u, np.zeros(hub, np.int32)])
+        v = np.concatenate([v, np.arange(1, hub + 1, dtype=np.int32)])
+        lo, hi = np.minimum(u, v).astype(np.int64), np.maximum(u, v).astype(np.int64)
+        _, first = np.unique(lo * n + hi, return_index=True)
+        u, v = u[first], v[first]
+        s = np.where(np.arange(len(u)) % 3 == 0, -1, 1).astype(np.int8)
+    g = O.clean_graph(n, u, v, s)
+    sb = P.SignedBal(0)
+    try:
+        sb.load_graph(n, u, v, s)
+        _check(P, sb, g, seed=n, t0=3, K=K)
+        sparse = synth.random_connected(40, 10, seed=5)
+        nv, _ = sb.load_batch([(n, u, v, s), sparse, (n, u, v, -s)])
+        sb.sample_trees_kruskal(n, 3, K)
+        counts, hashes = (x.cpu().numpy() for x in sb.batch_frustration())
+        for gi, r in enumerate([g, O.clean_graph(*sparse), O.clean_graph(n, u, v, -s)]):
+            ref = O.mst_sample(r, n, 3, K)
+            assert np.array_equal(counts[gi], ref["counts"]), gi
+            assert np.array_equal(hashes[gi].view(np.uint64), ref["hashes"]), gi
+    finally:
+        sb.close()
