@@ -106,7 +106,7 @@ sb_status sb_profile_read(sb_ctx* ctx, double* ms_out, int64_t* launches_out);
    SB_TUNE_SCORE_BLOCKS_SM   scorer blocks per SM (0 = as many as fit)
    SB_TUNE_GL_LANES          graphL lanes per row segment: 8 (32 columns),
                              16 (64 columns) or 32 (128 columns) when
-                             R % 4 == 0 (8)
+                             R % 4 == 0 (0 = the width that R suits)
    SB_TUNE_BFS_GROUP         lanes that share one vertex in the BFS, a power
                              of two in [1, 32]; used when it is at most twice
                              the launch's words rounded up to a power of two

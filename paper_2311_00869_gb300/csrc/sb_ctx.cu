@@ -236,6 +236,8 @@ void sb_release_graphl(sb_ctx* c)
     SB_FREE(gl_scale);
     SB_FREE(gl_colmax);
     SB_FREE(gl_misc);
+    SB_FREE(gl_signs);
+    c->gl_signs_cap = 0;
     if (c->gl_exec) cudaGraphExecDestroy(c->gl_exec);
     c->gl_exec = nullptr;
     memset(c->gl_exec_key, 0, sizeof(c->gl_exec_key));

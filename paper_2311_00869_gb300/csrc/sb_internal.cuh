@@ -183,6 +183,8 @@ struct sb_ctx {
     size_t gl_red_cap = 0;
     float* gl_buf = nullptr;       // ping-pong buffer for descent
     size_t gl_buf_cap = 0;
+    uint32_t* gl_signs = nullptr;  // sign words of one or two matrices
+    size_t gl_signs_cap = 0;
     float* gl_scale = nullptr;     // per-(graph, column) pending power-of-two scale
     size_t gl_scale_cap = 0;
     uint32_t* gl_colmax = nullptr;
@@ -202,7 +204,7 @@ struct sb_ctx {
 
     // captured descent loop (replayed while its arguments stay the same)
     cudaGraphExec_t gl_exec = nullptr;
-    uint64_t gl_exec_key[16] = {0};
+    uint64_t gl_exec_key[18] = {0};
     bool capturing = false;
     cudaStream_t cap_stream = nullptr;  // private stream: capture is not allowed on the legacy stream
     cudaEvent_t cap_in = nullptr, cap_out = nullptr;

@@ -3,6 +3,7 @@
 // graph and the tree's balanced state, lab[u] ^ lab[v] ^ neg summed per tree.
 #include <algorithm>
 
+#include "sb_count.cuh"
 #include "sb_internal.cuh"
 
 static int score_group_for(int Wb)
@@ -23,17 +24,7 @@ static int score_group_for(int Wb)
 // eights, flushed into 32-bit counts before the planes can overflow.
 #define SC_THREADS 256
 #define SC_TILE 2048                     // edges per shared-memory tile (16 KB)
-#define SC_PLANES 12                     // ripple planes of the eights
 #define SC_FAST_BATCH 1                  // whole 8-edge batches without per-edge checks
-#define SC_RIPPLE_EXIT 1                 // stop the ripple when no carry is left
-#define SC_FLUSH ((1 << SC_PLANES) - 1)  // batches of 8 edges between flushes
-
-__device__ __forceinline__ void csa(uint64_t& h, uint64_t& l, uint64_t a, uint64_t b, uint64_t c)
-{
-    const uint64_t u = a ^ b;
-    h = (a & b) | (u & c);
-    l = u ^ c;
-}
 
 struct ScoreArgs {
     const int2* edges;    // m edges + 2 of padding: (colder, hotter | neg << 31)
@@ -46,76 +37,6 @@ struct ScoreArgs {
     uint32_t* err;        // bit 0 set when a tile copy did not arrive in time
     long long wait;       // SM cycles a tile wait may take before it reports a timeout
     long long drain;      // SM cycles the copies still in flight get before a failed block exits
-};
-
-struct ScoreAcc {
-    uint64_t ones, twos, fours, P[SC_PLANES];
-    int nb;  // batches added since the last flush
-    __device__ __forceinline__ void reset()
-    {
-        ones = twos = fours = 0;
-#pragma unroll
-        for (int b = 0; b < SC_PLANES; b++) P[b] = 0;
-        nb = 0;
-    }
-    __device__ __forceinline__ void add8(const uint64_t* x)
-    {
-        uint64_t twosA, twosB, foursA, foursB, eights;
-        csa(twosA, ones, ones, x[0], x[1]);
-        csa(twosB, ones, ones, x[2], x[3]);
-        csa(foursA, twos, twos, twosA, twosB);
-        csa(twosA, ones, ones, x[4], x[5]);
-        csa(twosB, ones, ones, x[6], x[7]);
-        csa(foursB, twos, twos, twosA, twosB);
-        csa(eights, fours, fours, foursA, foursB);
-        uint64_t cy = eights;
-#pragma unroll
-        for (int b = 0; b < SC_PLANES; b++) {
-            if (SC_RIPPLE_EXIT && !cy) break;  // carries die out after a few planes
-            const uint64_t t = P[b] & cy;
-            P[b] ^= cy;
-            cy = t;
-        }
-        nb++;
-    }
-    __device__ __forceinline__ uint32_t count(int t) const
-    {
-        uint32_t hi = 0;
-#pragma unroll
-        for (int b = 0; b < SC_PLANES; b++) {
-            if (!(nb >> b)) break;  // nb batches hold at most nb eights
-            hi |= (uint32_t)((P[b] >> t) & 1ull) << b;
-        }
-        return 8u * hi + 4u * (uint32_t)((fours >> t) & 1ull) + 2u * (uint32_t)((twos >> t) & 1ull) +
-               (uint32_t)((ones >> t) & 1ull);
-    }
-    // adds the 64 counters into dst[0..63] (shared or global memory)
-    __device__ __forceinline__ void flush(uint32_t* dst)
-    {
-        if (nb == 0) return;
-        for (int t = 0; t < 64; t++) {
-            const uint32_t val = count(t);
-            if (val) atomicAdd(dst + t, val);
-        }
-        reset();
-    }
-    // the same for a whole warp whose lanes gl, gl + G, .. hold counters of one
-    // word (dst; lanes with `act` false hold none): those lanes are summed
-    // first, and the lanes of different words start at different trees, so that
-    // their atomics fall in different banks (16 words, 1 M edges: 60 -> 48 us
-    // for the kernel, most of it this flush)
-    template <int G>
-    __device__ __forceinline__ void flush_warp(uint32_t* dst, bool act)
-    {
-        const int gl = (int)(threadIdx.x & (G - 1));
-        for (int i = 0; i < 64; i++) {
-            const int t = (i + gl) & 63;
-            uint32_t val = act ? count(t) : 0u;
-#pragma unroll
-            for (int d = G; d < 32; d <<= 1) val += __shfl_xor_sync(0xffffffffu, val, d);
-            if (val && (threadIdx.x & 31) < G) atomicAdd(dst + t, val);
-        }
-    }
 };
 
 template <int G, bool SEG>
@@ -199,7 +120,7 @@ __global__ void __launch_bounds__(SC_THREADS, SEG ? 3 : 4) k_score(ScoreArgs A)
                                            (ed[k].y < 0 ? ~0ull : 0ull))
                                         : 0ull;
                 if (SEG) {
-                    // edges are sorted by graph: split the batch into runs of one graph
+                    // edges are sorted by graph
                     int32_t gk[8];
                     uint32_t rem = 0;
 #pragma unroll
@@ -207,25 +128,7 @@ __global__ void __launch_bounds__(SC_THREADS, SEG ? 3 : 4) k_score(ScoreArgs A)
                         gk[k] = ed[k].x >= 0 ? A.vgid[ed[k].x] : -1;
                         rem |= (ed[k].x >= 0 ? 1u : 0u) << k;
                     }
-                    while (rem) {
-                        int32_t g = -1;
-#pragma unroll
-                        for (int k = 7; k >= 0; k--)
-                            if ((rem >> k) & 1u) g = gk[k];  // graph of the first remaining edge
-                        uint64_t xm[8];
-#pragma unroll
-                        for (int k = 0; k < 8; k++) {
-                            const bool tk = ((rem >> k) & 1u) && gk[k] == g;
-                            xm[k] = tk ? x[k] : 0ull;
-                            if (tk) rem &= ~(1u << k);
-                        }
-                        if (g != gcur) {
-                            if (gcur >= 0) acc.flush(dst0 + gcur * A.KP);
-                            gcur = g;
-                        }
-                        acc.add8(xm);
-                        if (acc.nb == SC_FLUSH) acc.flush(dst0 + gcur * A.KP);
-                    }
+                    acc.add8_runs(x, gk, rem, gcur, dst0, A.KP);
                     continue;
                 } else {
                     acc.add8(x);
@@ -246,7 +149,7 @@ __global__ void __launch_bounds__(SC_THREADS, SEG ? 3 : 4) k_score(ScoreArgs A)
     }
     if (SEG && act && gcur >= 0) acc.flush(dst0 + gcur * A.KP);
     if (!SEG) {
-        acc.template flush_warp<G>(dst0, act);
+        acc.template flush_warp<G>(scnt + 64 * 32 * slice);
         __syncthreads();
         for (int i = tid; i < A.Wb * 64; i += SC_THREADS)
             if (scnt[i]) atomicAdd(A.counts + 64 * A.w0 + i, scnt[i]);
