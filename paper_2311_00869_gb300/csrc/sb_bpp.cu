@@ -3,35 +3,68 @@
 // restated with Harary's bipartition, Sec. 2), the state hash that keys the
 // frustration cloud (the frustration scorer is in sb_score.cu).
 //
-// Data layout (vertex-major, 64 trees per uint64 word):
-//   labels[v * W + w]  bit b = parity label of tree 64 w + b at vertex v
-//   vis / frontier     [v * Wb + w] for the Wb words of one BFS launch
+// Data layout (vertex-major, 32 trees per half-word, 64 per uint64 word):
+//   labels[v * W + w]  bit b = parity label of slot 64 w + b at vertex v
+//   vis / frontier     [v * H + h] for the H half-words of one BFS launch
+// A slot holds one tree of the batch (k_tree_order says which).
+//
 // A BFS launch grows up to 32 words (2048 trees) at once, level by level, in
-// one cooperative persistent kernel: a group of G lanes owns one vertex (lane
-// = word), gathers its neighbours' frontier words with coalesced row loads,
-// and picks each newly reached tree's parent as the argmin of the packed key
-// (fmix32((u ^ y_v) + a_t) << 32 | u).  fmix32 is a bijection, so the hash
-// alone orders the candidates of one (tree, vertex): comparing 32-bit hashes
-// is the 64-bit packed argmin.  Rows longer than SB_BFS_CHUNK are split over
-// several groups that merge with 64-bit atomicMin on the packed key.
+// one cooperative persistent kernel: a group of G lanes owns one vertex (or one
+// slice of 32 half-words of it), lane = half-word, gathers its neighbours'
+// frontier rows with coalesced loads, and picks each newly reached tree's
+// parent as the argmin of the packed key (fmix32((u ^ y_v) + a_t) << 32 | u).
+// fmix32 is a bijection, so the hash alone orders the candidates of one (tree,
+// vertex): comparing 32-bit hashes is the 64-bit packed argmin.  Rows longer
+// than SB_BFS_CHUNK are split over several groups that merge with 64-bit
+// atomicMin on the packed key.
+//
+// What bounds it: instructions of the hash loop (on the 2^20 R-MAT graph with
+// 1024 trees 13.0 G warp instructions for 6.8 G candidates, 74 % of the issue
+// slots, the ALU pipe 71 % busy; on the 2^24 graph also the frontier rows from
+// DRAM).  A lane walks its own candidates, so what counts is that the lanes of
+// a warp have about as many each.  One lane per half-word puts one vertex into
+// a warp from 16 words on (one lane per 64-tree word made that two, whose
+// neighbours differ), trees are dealt out over the
+// half-words by depth, and warps take their work items as they get free instead
+// of waiting for the slowest at every level.  With those shares so even, a
+// queue that rebalances a tile's candidates over the group costs more than it
+// gives in a whole warp (17.4 against 18.4 ms) and stays for narrower groups,
+// whose vertices differ (45 against 62 ms on 512 uneven graphs).
 #include <algorithm>
 
 #include "sb_internal.cuh"
 
+// Work items are sorted by degree.  Whole-warp groups: one round of items is
+// dealt out in advance, the next BFS_SINGLE_PCT per cent of them are taken one
+// by one and the rest, light by then, A.grab at a time.  All dealt out in
+// advance (a round of one per group, the order reversing every round): 17.4 /
+// 616 ms (2^20, 2^24 graph); half of them 16.8 / 571, a tenth 14.8 / 524; as
+// here 13.9 / 506 (30 per cent one by one 14.2 / 523, everything 14.7 / 570: a
+// ticket is an atomic on one counter).  Narrower groups: BFS_FIXED_PCT per cent
+// in advance, the rest 4 per group and ticket (39.2 ms on 512 uneven graphs,
+// 43.2 all in advance).
+#define BFS_SINGLE_PCT 10
+#define BFS_FIXED_PCT 40
 #define BFS_THREADS 128
 #define BFS_THREADS_PAR 128
-// Candidate-queue entries per lane (overflow falls back to per-lane hashing):
-// the host takes the largest count in this range that keeps the most blocks
-// resident per SM (the salts of a launch grow with its words).
-#define BFS_QUEUE_MIN 8
-#define BFS_QUEUE_MAX 32
-#define BFS_BLOCKS_PER_SM 5     // the registers of one block allow 5 per SM (at most 102 per thread)
+// Candidate-queue entries per lane (more are hashed lane by lane).
+#define BFS_QUEUE 16
+// 28 warps, 72 registers: 588 ms per 4096 trees on the 2^24 graph, 627 with 6
+// blocks (85 registers) and 602 with 8 (64); 16.6 / 16.7 / 16.7 ms per 1024
+// trees on the 2^20 graph.
+#define BFS_BLOCKS_PER_SM 7
+// Batches on graphs of at least this many vertices fill the slots by the
+// trees' expected depth: 589 -> 506 ms per 4096 trees on the 2^24 graph, 14.6 ->
+// 13.9 ms per 1024 on the 2^20 graph, 1.45 -> 1.42 ms at 95,000 vertices, where
+// bringing the labels back into tree order takes about as much.
+#define BFS_ORDER_MIN (1 << 18)
+// Threads per SM below which a launch spreads its half-words over more lanes.
+#define BFS_SPREAD_THREADS 512
 #define SYNC_WORDS 48
-// Shared-memory slots of (owner thread o, tree t): owner-major rows padded so
-// that one owner's trees, and one tree of consecutive owners, fall in
-// different banks (the hash rounds walk one owner's trees in lockstep).
-#define BSLOT(o, t) ((o) * 65 + (t))  // 32-bit minima / winner ids
-#define KSLOT(w, t) ((w) * 65 + (t))  // tree salts of word w
+// Shared-memory slots: rows of one owner thread's 32 trees (running minima,
+// winner ids), 16-byte aligned, and of one half-word's tree salts.
+#define BSLOT(o, t) ((o) * 36 + (t))
+#define KSLOT(h, t) ((h) * 33 + (t))
 
 struct BfsArgs {
     const sb_bfs_item* items;
@@ -39,23 +72,29 @@ struct BfsArgs {
     const int32_t* col;
     const int32_t* hub_vertex;
     int64_t n_hubs;
-    uint64_t* lab;   // n x Wt
-    int Wt, w0, Wb;
-    uint64_t* vis;   // n x Wb
-    uint64_t* fr0;
-    uint64_t* fr1;
-    int32_t* done;
-    uint64_t* hubnew;   // n_hubs x Wb
-    uint64_t* hubbest;  // n_hubs x Wb x 64
+    uint32_t* lab;      // n x Ht half-words
+    int Ht, h0;         // half-words of the batch; first one of this launch
+    int H;              // half-words of this launch
+    int slices;         // groups of 32 half-words, 1 or 2
+    int64_t fixed_rounds;    // rounds of units dealt out in advance; the rest are taken as warps get free,
+    int64_t single_tickets;  // that many times one unit per group, then
+    int grab;                // `grab` units per group at a time
+    int ls;             // 1 << ls lanes share a half-word, 32 >> ls trees each
+    uint32_t* vis;      // n x H
+    uint32_t* fr0;
+    uint32_t* fr1;
+    int32_t* done;      // n x slices: level at which every tree had the vertex, or -1
+    uint32_t* hubnew;   // n_hubs x H
+    uint64_t* hubbest;  // n_hubs x H x 32
     uint32_t* sync;
     int32_t* parents;   // K x n or null
     int64_t n;
-    uint64_t S;         // seed key
+    uint64_t S;            // seed key
     const int64_t* tree0;  // global index of batch tree 0 (device)
+    const int32_t* perm;   // tree of each slot, or null (slot = tree)
     const int32_t* vgoff;  // first vertex of each vertex's graph (batches), or null
     long long wait;        // SM cycles a barrier wait may take before it reports a timeout
     unsigned bar_extra;    // arrivals a barrier expects beyond the launch's blocks (0; 1 tests the timeout path)
-    int qcap;              // candidate-queue entries per lane
 };
 
 // ----------------------------------------------------------- grid barrier
@@ -96,19 +135,14 @@ __device__ __forceinline__ unsigned group_mask(int G)
     return ((1u << G) - 1u) << base;
 }
 
-// Fetch the 128-byte line at p into L2 (no register result, nothing waits).
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
-// Winner label bits: each lane keeps its trees' bits in two registers (trees
-// 0-31 and 32-63) while it hashes its own candidates; the queue paths, where
-// lanes write each other's trees, work on a copy in shared memory (two words
-// per thread) with atomic bit updates.
+// Winner label bits: each lane keeps its trees' bits in a register while it
+// hashes its own candidates; the queue path, where lanes write each other's
+// trees, works on a copy in shared memory with atomic bit updates.
 __device__ __forceinline__ void lbit_put_atomic(uint32_t* lbits, int o, int t, uint32_t v)
 {
-    uint32_t* w = lbits + 2 * o + (t >> 5);
-    const uint32_t m = 1u << (t & 31);
-    if (v) atomicOr(w, m);
-    else atomicAnd(w, ~m);
+    const uint32_t m = 1u << t;
+    if (v) atomicOr(lbits + o, m);
+    else atomicAnd(lbits + o, ~m);
 }
 
 // Position of the highest set bit of a nonzero word.
@@ -133,218 +167,221 @@ __device__ __forceinline__ int group_excl_scan(int x, unsigned gmask, int gl, in
     return incl - x;
 }
 
-// One pass over a CSR range for one vertex: lane gl of the group owns word
-// w0 + gl.  Neighbours are read 8 at a time so that 8 frontier gathers are in
-// flight per lane.  It keeps the running argmin of the hashed parent key over
-// the candidates in `mask`: best (initialised to 0xFFFFFFFF) holds the
-// smallest hash, lbv / bestu the winner's label bit / id; keys are distinct
-// (the hash is a bijection in u), so `h <= best` accepts exactly the minimum.
-// `once` returns the trees that had a candidate.  For each tile of 8
-// neighbours the lanes hash their own candidates when their shares are even;
-// otherwise the group's candidate bits are compacted into a shared queue
-// (entry = neighbour, owner lane, tree, label bit) and hashed by all lanes in
-// lockstep: the 8 neighbours at once (atomicMin, then the entry equal to the
-// minimum writes its label), or, when they hold more candidates than the
-// queue, one neighbour at a time (its entries have distinct slots).
-// `cur` and `lab` are rewritten between levels by other blocks, so they are
-// read with plain (coherent) loads; the column array is read-only.
-template <bool PAR, int BD, int G>
-__device__ __forceinline__ void scan_row(const int32_t* cp, int len, const uint64_t* cur, const uint64_t* lab, int Wb,
-                                         int Wt, int wofs, int gl, uint64_t mask, uint32_t y, uint32_t goff,
-                                         const uint32_t* akey, uint32_t* best, uint32_t* lbits, uint32_t (&lbv)[2],
-                                         int32_t* bestu, uint16_t* queue, int qcap, uint32_t* hxs, int tid, unsigned gmask,
-                                         uint64_t& once, uint32_t& nhash)
+// Hashes one lane's candidates m of neighbour u (label word lw), two at a time
+// (the highest and the lowest: the same one when a single candidate is left,
+// whose second update then repeats the first).
+template <bool PAR>
+__device__ __forceinline__ void hash_candidates(uint32_t m, uint32_t lw, uint32_t u, uint32_t y, const uint32_t* ak,
+                                                uint32_t* bs, uint32_t& lbv, int32_t* bu)
 {
-    // frontier rows are Wb words (128 B at 16 words) at 8 Wb-byte offsets; the
-    // rows of the tile after next are fetched into L2 while this tile is
-    // hashed, one line per lane (lanes 0-7: first lines of the 8 rows, lanes
-    // 8-15: second lines)
-    const int pf_k = gl & 7, pf_line = gl >> 3;
-    const bool pf = gl < 16 && pf_line * 16 < Wb;
-    for (int j = 0; j < len; j += 8) {
-        uint32_t c[8];
-        uint64_t f[8], l[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) c[k] = (j + k < len) ? (uint32_t)__ldg(cp + j + k) : 0u;
-        if (pf && j + 16 + pf_k < len) {
-            const uint32_t cn = (uint32_t)__ldg(cp + j + 16 + pf_k);
-            prefetch_l2(cur + (int64_t)(cn & SB_ID_MASK) * Wb + 16 * pf_line);
+    const uint32_t hx = u ^ y;
+    while (m) {
+        const int ia = bit_high(m);
+        const int ib = __ffs((int)m) - 1;
+        const uint32_t bita = 1u << ia, bitb = 1u << ib;
+        m &= ~(bita | bitb);
+        const uint32_t ha = sb_fmix32(hx + ak[ia]);
+        const uint32_t hb = sb_fmix32(hx + ak[ib]);
+        const uint32_t ba = bs[ia], bb = bs[ib];
+        if (ha <= ba) {  // <=: the minima start at 0xFFFFFFFF
+            bs[ia] = ha;
+            lbv ^= (lbv ^ lw) & bita;  // the winner's label bit
+            if (PAR) bu[ia] = (int32_t)u;
         }
-#pragma unroll
-        for (int k = 0; k < 8; k++)
-            f[k] = (j + k < len && mask) ? (cur[(int64_t)(c[k] & SB_ID_MASK) * Wb + gl] & mask) : 0ull;
-#pragma unroll
-        for (int k = 0; k < 8; k++)
-            l[k] = f[k] ? (lab[(int64_t)(c[k] & SB_ID_MASK) * Wt + wofs] ^ ((c[k] >> 31) ? ~0ull : 0ull)) : 0ull;
-        {
-            const int owner0 = tid - gl;  // thread index of the group's lane 0
-            int cnt = 0;
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                once |= f[k];
-                cnt += __popcll(f[k]);
-            }
-            const unsigned Tsum = __reduce_add_sync(gmask, (unsigned)cnt);
-            if (Tsum == 0) continue;  // same for the whole group
-            nhash += (uint32_t)cnt;
-            const unsigned cmax = __reduce_max_sync(gmask, (unsigned)cnt);
-            if (cmax * G <= 2 * Tsum + 2 * G) {
-                // the lanes' shares are even enough: every lane hashes its own
-                // candidates into its own slots (32-bit halves, two at a time),
-                // with no queue and no synchronisation
-                const uint32_t* ak = akey + KSLOT(gl, 0);
-                uint32_t* bs = best + BSLOT(tid, 0);
-#pragma unroll
-                for (int k = 0; k < 8; k++) {
-                    const uint32_t u = (c[k] & SB_ID_MASK) - goff;
-                    const uint32_t hx = u ^ y;
-#pragma unroll
-                    for (int half = 0; half < 2; half++) {
-                        uint32_t m = (uint32_t)(f[k] >> (32 * half));
-                        const uint32_t lw = (uint32_t)(l[k] >> (32 * half));
-                        const int t0 = 32 * half;
-                        while (m) {
-                            // the highest and the lowest candidate (the same
-                            // one when a single candidate is left)
-                            const int ia = bit_high(m);
-                            const int ib = __ffs(m) - 1;
-                            const bool two = ia != ib;
-                            m &= ~((1u << ia) | (1u << ib));
-                            const uint32_t ha = sb_fmix32(hx + ak[t0 + ia]);
-                            const uint32_t hb = sb_fmix32(hx + ak[t0 + ib]);
-                            const uint32_t ba = bs[t0 + ia], bb = bs[t0 + ib];
-                            // the winner's label bit goes into bit t of the half's label word
-                            if (ha <= ba) {  // <=: the minima start at 0xFFFFFFFF
-                                bs[t0 + ia] = ha;
-                                lbv[half] ^= (lbv[half] ^ lw) & (1u << ia);
-                                if (PAR) bestu[BSLOT(tid, t0 + ia)] = (int32_t)u;
-                            }
-                            if (two && hb <= bb) {
-                                bs[t0 + ib] = hb;
-                                lbv[half] ^= (lbv[half] ^ lw) & (1u << ib);
-                                if (PAR) bestu[BSLOT(tid, t0 + ib)] = (int32_t)u;
-                            }
-                        }
-                    }
-                }
-                continue;
-            }
-            // the queue paths update other lanes' label bits: through shared memory
-            lbits[2 * tid] = lbv[0];
-            lbits[2 * tid + 1] = lbv[1];
-            int T;
-            int pos = group_excl_scan<G>(cnt, gmask, gl, T);
-            if (T <= qcap * G) {
-                // the candidates of all 8 neighbours go through one queue of
-                // (neighbour, owner word, tree, label bit) entries; lanes hash
-                // them in lockstep, keep each tree's minimum with atomicMin
-                // (two neighbours may reach the same tree) and then let the
-                // one entry equal to the minimum write its label bit
-#pragma unroll
-                for (int k = 0; k < 8; k++) {
-                    // the group's table of the 8 neighbours' u ^ y (one writer per entry)
-                    if ((k & (G - 1)) == gl) hxs[k] = ((c[k] & SB_ID_MASK) - goff) ^ y;
-                    for (uint64_t b = f[k]; b;) {
-                        const int t = __ffsll((long long)b) - 1;
-                        b &= b - 1;
-                        queue[pos++] = (uint16_t)((k << 12) | (gl << 7) | (t << 1) | (int)((l[k] >> t) & 1ull));
-                    }
-                }
-                __syncwarp(gmask);
-                for (int i = gl; i < T; i += G) {
-                    const uint32_t e = queue[i];
-                    const int k = (int)(e >> 12), ow = (int)((e >> 7) & 31u), t = (int)((e >> 1) & 63u);
-                    const uint32_t h = sb_fmix32(hxs[k] + akey[KSLOT(ow, t)]);
-                    atomicMin(&best[BSLOT(owner0 + ow, t)], h);
-                }
-                __syncwarp(gmask);
-                for (int i = gl; i < T; i += G) {
-                    const uint32_t e = queue[i];
-                    const int k = (int)(e >> 12), ow = (int)((e >> 7) & 31u), t = (int)((e >> 1) & 63u);
-                    const uint32_t hxk = hxs[k];
-                    const uint32_t h = sb_fmix32(hxk + akey[KSLOT(ow, t)]);
-                    const uint32_t u = hxk ^ y;
-                    const int o = owner0 + ow;
-                    if (best[BSLOT(o, t)] == h) {  // fmix32 is injective in u: one entry matches
-                        lbit_put_atomic(lbits, o, t, e & 1u);
-                        if (PAR) bestu[BSLOT(o, t)] = (int32_t)u;
-                    }
-                }
-                __syncwarp(gmask);
-                lbv[0] = lbits[2 * tid];
-                lbv[1] = lbits[2 * tid + 1];
-                continue;
-            }
-            // many candidates: one neighbour at a time
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                const int cntk = __popcll(f[k]);
-                int Tk;
-                int posk = group_excl_scan<G>(cntk, gmask, gl, Tk);
-                if (Tk == 0) continue;  // same for the whole group
-                const uint32_t u = (c[k] & SB_ID_MASK) - goff;  // id inside the graph
-                const uint32_t hx = u ^ y;
-                if (Tk > qcap * G) {
-                    // more candidates than the queue holds; each lane hashes
-                    // its own bits (it alone owns their slots)
-                    for (uint64_t b = f[k]; b;) {
-                        const int t = __ffsll((long long)b) - 1;
-                        b &= b - 1;
-                        const uint32_t h = sb_fmix32(hx + akey[KSLOT(gl, t)]);
-                        if (h <= best[BSLOT(tid, t)]) {  // <=: the minima start at 0xFFFFFFFF
-                            best[BSLOT(tid, t)] = h;
-                            lbit_put_atomic(lbits, tid, t, (uint32_t)(l[k] >> t) & 1u);
-                            if (PAR) bestu[BSLOT(tid, t)] = (int32_t)u;
-                        }
-                    }
-                    __syncwarp(gmask);
-                    continue;
-                }
-                for (uint64_t b = f[k]; b;) {
-                    const int t = __ffsll((long long)b) - 1;
-                    b &= b - 1;
-                    queue[posk++] = (uint16_t)((gl << 7) | (t << 1) | (int)((l[k] >> t) & 1ull));
-                }
-                __syncwarp(gmask);
-                // two entries per lane and round: entries of one neighbour have
-                // distinct slots, so their updates are independent
-                for (int i = gl; i < Tk; i += 2 * G) {
-                    const bool two = i + G < Tk;
-                    const uint32_t ea = queue[i], eb = queue[two ? i + G : i];
-                    const int owa = (int)((ea >> 7) & 31u), ta = (int)((ea >> 1) & 63u);
-                    const int owb = (int)((eb >> 7) & 31u), tb = (int)((eb >> 1) & 63u);
-                    const uint32_t ha = sb_fmix32(hx + akey[KSLOT(owa, ta)]);
-                    const uint32_t hb = sb_fmix32(hx + akey[KSLOT(owb, tb)]);
-                    const int oa = owner0 + owa, ob = owner0 + owb;
-                    const uint32_t ba = best[BSLOT(oa, ta)], bb = best[BSLOT(ob, tb)];
-                    if (ha <= ba) {
-                        best[BSLOT(oa, ta)] = ha;
-                        lbit_put_atomic(lbits, oa, ta, ea & 1u);
-                        if (PAR) bestu[BSLOT(oa, ta)] = (int32_t)u;
-                    }
-                    if (two && hb <= bb) {
-                        best[BSLOT(ob, tb)] = hb;
-                        lbit_put_atomic(lbits, ob, tb, eb & 1u);
-                        if (PAR) bestu[BSLOT(ob, tb)] = (int32_t)u;
-                    }
-                }
-                __syncwarp(gmask);
-            }
-            lbv[0] = lbits[2 * tid];
-            lbv[1] = lbits[2 * tid + 1];
+        if (hb <= bb) {
+            bs[ib] = hb;
+            lbv ^= (lbv ^ lw) & bitb;
+            if (PAR) bu[ib] = (int32_t)u;
         }
     }
 }
 
-// Resets the running minima of the trees in `mask`.
-template <int BD>
-__device__ __forceinline__ void best_reset(uint32_t* best, int tid, uint64_t mask)
+// scan_row for a whole warp per vertex: its lanes look at the same neighbour
+// and, with the trees dealt out evenly over the half-words, hold about as many
+// candidates each, so every lane hashes its own.
+template <bool PAR>
+__device__ __forceinline__ void scan_row_warp(const int32_t* cp, int len, const uint32_t* cur, const uint32_t* lab, int H,
+                                              int Ht, uint32_t mask, uint32_t y, uint32_t goff, const uint32_t* ak,
+                                              uint32_t* bs, uint32_t& lbv, int32_t* bu, uint32_t& once, uint32_t& nhash)
 {
-    for (uint64_t b = mask; b;) {
-        const int t = __ffsll((long long)b) - 1;
-        b &= b - 1;
-        best[BSLOT(tid, t)] = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const bool any_mask = mask != 0;
+    uint32_t cols = 0;
+    for (int j = 0; j < len; j += 8) {
+        uint32_t c[8], f[8];
+        if ((j & 31) == 0) cols = j + lane < len ? (uint32_t)__ldg(cp + j + lane) : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; k++) c[k] = __shfl_sync(0xffffffffu, cols, (j & 31) + k);
+#pragma unroll
+        for (int k = 0; k < 8; k++) f[k] = 0;
+        if (any_mask) {
+            if (j + 8 <= len) {
+#pragma unroll
+                for (int k = 0; k < 8; k++) f[k] = cur[(int64_t)(c[k] & SB_ID_MASK) * H];
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; k++)
+                    if (j + k < len) f[k] = cur[(int64_t)(c[k] & SB_ID_MASK) * H];
+            }
+        }
+        uint32_t any = 0;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            f[k] &= mask;
+            any |= f[k];
+        }
+        if (!__any_sync(0xffffffffu, any != 0)) continue;
+        once |= any;
+        uint32_t l[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            l[k] = 0;
+            if (f[k]) l[k] = lab[(int64_t)(c[k] & SB_ID_MASK) * Ht];
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            nhash += (uint32_t)__popc(f[k]);
+            hash_candidates<PAR>(f[k], l[k] ^ (uint32_t)((int32_t)c[k] >> 31), (c[k] & SB_ID_MASK) - goff, y, ak, bs,
+                                 lbv, bu);
+        }
     }
+}
+
+// One pass over a CSR range for one vertex: lane gl of the group owns the
+// trees in its `mask` of one half-word.  Neighbours are read 8 at a time so
+// that 8 frontier gathers are in flight per lane.  It keeps the running argmin
+// of the hashed parent key over the candidates: best (initialised to
+// 0xFFFFFFFF) holds the smallest hash, lbv / bestu the winner's label bit /
+// id; keys are distinct (the hash is a bijection in u), so `h <= best` accepts
+// exactly the minimum.  `once` returns the trees that had a candidate.  For
+// each tile of 8 neighbours the lanes hash their own candidates when their
+// shares are even; otherwise the group's candidate bits are compacted into a
+// shared queue (entry = neighbour, owner lane, tree, label bit) and hashed by
+// all lanes in lockstep (atomicMin, then the entry equal to the minimum writes
+// its label).
+// `cur` and `lab` are rewritten between levels by other blocks, so they are
+// read with plain (coherent) loads; the column array is read-only.
+template <bool PAR, int G>
+__device__ __forceinline__ void scan_row(const int32_t* cp, int len, const uint32_t* cur, const uint32_t* lab, int H,
+                                         int Ht, int gl, int ls, uint32_t mask, uint32_t y, uint32_t goff,
+                                         const uint32_t* akey, const uint32_t* ak, uint32_t* best, uint32_t* lbits,
+                                         uint32_t& lbv, int32_t* bestu, uint16_t* queue, uint32_t* hxs, int tid,
+                                         unsigned gmask, uint32_t& once, uint32_t& nhash)
+{
+    uint32_t* const bs = best + BSLOT(tid, 0);
+    const int owner0 = tid - gl;  // thread index of the group's lane 0
+    for (int j = 0; j < len; j += 8) {
+        uint32_t c[8], f[8], l[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) c[k] = (j + k < len) ? (uint32_t)__ldg(cp + j + k) : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; k++) f[k] = (j + k < len && mask) ? (cur[(int64_t)(c[k] & SB_ID_MASK) * H] & mask) : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            l[k] = f[k] ? (lab[(int64_t)(c[k] & SB_ID_MASK) * Ht] ^ (uint32_t)((int32_t)c[k] >> 31)) : 0u;
+        int cnt = 0;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            once |= f[k];
+            cnt += __popc(f[k]);
+        }
+        const unsigned Tsum = __reduce_add_sync(gmask, (unsigned)cnt);
+        if (Tsum == 0) continue;  // same for the whole group
+        nhash += (uint32_t)cnt;
+        const unsigned cmax = __reduce_max_sync(gmask, (unsigned)cnt);
+        if (cmax * G <= 4 * Tsum + 2 * G || Tsum > BFS_QUEUE * G) {
+            // the lanes' shares are even enough (or too many to queue): every
+            // lane hashes its own candidates into its own slots, two at a
+            // time, with no queue and no synchronisation
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                hash_candidates<PAR>(f[k], l[k], (c[k] & SB_ID_MASK) - goff, y, ak, bs, lbv,
+                                     PAR ? bestu + BSLOT(tid, 0) : nullptr);
+            continue;
+        }
+        // the queue path updates other lanes' label bits: through shared memory
+        lbits[tid] = lbv;
+        int T;
+        int pos = group_excl_scan<G>(cnt, gmask, gl, T);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            // the group's table of the 8 neighbours' u ^ y (one writer per entry)
+            if ((k & (G - 1)) == gl) hxs[k] = ((c[k] & SB_ID_MASK) - goff) ^ y;
+            for (uint32_t b = f[k]; b;) {
+                const int t = __ffs((int)b) - 1;
+                b &= b - 1;
+                queue[pos++] = (uint16_t)((k << 12) | (gl << 7) | (t << 1) | (int)((l[k] >> t) & 1u));
+            }
+        }
+        __syncwarp(gmask);
+        for (int i = gl; i < T; i += G) {
+            const uint32_t e = queue[i];
+            const int k = (int)(e >> 12), ow = (int)((e >> 7) & 31u), t = (int)((e >> 1) & 31u);
+            atomicMin(&best[BSLOT(owner0 + ow, t)], sb_fmix32(hxs[k] + akey[KSLOT(ow >> ls, t)]));
+        }
+        __syncwarp(gmask);
+        for (int i = gl; i < T; i += G) {
+            const uint32_t e = queue[i];
+            const int k = (int)(e >> 12), ow = (int)((e >> 7) & 31u), t = (int)((e >> 1) & 31u);
+            const uint32_t hxk = hxs[k];
+            const uint32_t h = sb_fmix32(hxk + akey[KSLOT(ow >> ls, t)]);
+            const int o = owner0 + ow;
+            if (best[BSLOT(o, t)] == h) {  // fmix32 is injective in u: one entry matches
+                lbit_put_atomic(lbits, o, t, e & 1u);
+                if (PAR) bestu[BSLOT(o, t)] = (int32_t)(hxk ^ y);
+            }
+        }
+        __syncwarp(gmask);
+        lbv = lbits[tid];
+    }
+}
+
+// Phase B of one level for one split row: the merged minima of its chunks
+// (a warp; lane = half-word, then lane = tree).
+template <bool PAR>
+__device__ __forceinline__ bool bfs_hub(const BfsArgs& A, int L, uint32_t* nxt, int64_t hi, int sl)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t v = A.hub_vertex[hi];
+    const int64_t dslot = (int64_t)v * A.slices + sl;
+    const int32_t d = A.done[dslot];
+    if (d >= 0 && L >= d + 3) return false;
+    const int h = 32 * sl + lane;
+    const bool act = h < A.H;
+    uint32_t visw = ~0u, nw = 0, labw = 0;
+    if (act) {
+        visw = A.vis[(int64_t)v * A.H + h];
+        nw = A.hubnew[hi * A.H + h] & ~visw;
+        A.hubnew[hi * A.H + h] = 0;
+    }
+    for (uint32_t hs = __ballot_sync(0xffffffffu, nw != 0); hs; hs &= hs - 1) {
+        const int hh = __ffs((int)hs) - 1;
+        const uint32_t w = __shfl_sync(0xffffffffu, nw, hh);
+        uint64_t key = 0;
+        if ((w >> lane) & 1u) {
+            uint64_t* hb = A.hubbest + (hi * A.H + 32 * sl + hh) * 32 + lane;
+            key = *hb;
+            *hb = ~0ull;
+            if (PAR && A.parents) {
+                const int64_t slot = 32 * (int64_t)(A.h0 + 32 * sl + hh) + lane;
+                A.parents[(A.perm ? (int64_t)A.perm[slot] : slot) * A.n + v] = (int32_t)((key >> 1) & SB_ID_MASK);
+            }
+        }
+        const uint32_t lb = __ballot_sync(0xffffffffu, (key & 1ull) != 0);
+        if (lane == hh) labw = lb;
+    }
+    if (act) {
+        if (nw) {
+            if (labw) A.lab[(int64_t)v * A.Ht + A.h0 + h] |= labw;
+            A.vis[(int64_t)v * A.H + h] = visw | nw;
+        }
+        nxt[(int64_t)v * A.H + h] = nw;
+    }
+    if (d < 0) {
+        const bool all = __all_sync(0xffffffffu, (visw | nw) == ~0u);
+        if (all && lane == 0) A.done[dslot] = L;
+    }
+    return nw != 0;
 }
 
 template <int G, bool PAR>
@@ -352,151 +389,160 @@ __global__ void __launch_bounds__(PAR ? BFS_THREADS_PAR : BFS_THREADS, PAR ? 2 :
     k_bfs(BfsArgs A)
 {
     constexpr int BD = PAR ? BFS_THREADS_PAR : BFS_THREADS;
-    extern __shared__ uint32_t smem[];
-    uint32_t* akey = smem;                        // tree salts, KSLOT(word, tree)
-    uint32_t* best = smem + A.Wb * 65;            // running minima, BSLOT(thread, tree)
-    uint32_t* lbits = best + 65 * BD;             // winners' label bits (queue paths), two words per thread
-    uint16_t* queues = (uint16_t*)(lbits + 2 * BD);  // A.qcap x G entries per group
-    int32_t* bestu = (int32_t*)(queues + ((A.qcap * BD + 1) & ~1));  // winners, BSLOT (PAR only)
-    uint32_t* hx_tab = (uint32_t*)(bestu + (PAR ? 65 * BD : 0));    // 8 neighbours' u ^ y per group
+    extern __shared__ __align__(16) uint32_t smem[];
+    uint32_t* best = smem;                            // running minima, BSLOT(thread, tree)
+    uint32_t* akey = best + BSLOT(BD, 0);             // tree salts, KSLOT(half-word, tree)
+    uint32_t* lbits = akey + A.H * 33;                // winners' label bits (queue path)
+    uint32_t* hx_tab = lbits + BD;                    // 8 neighbours' u ^ y per group
+    int32_t* bestu = (int32_t*)(hx_tab + 8 * (BD / G));  // winners, BSLOT (PAR only)
+    uint16_t* queues = (uint16_t*)(bestu + (PAR ? BSLOT(BD, 0) : 0));  // BFS_QUEUE x G entries per group
     __shared__ uint32_t s_any, s_stop;
 
     const int tid = threadIdx.x;
     const int gl = tid & (G - 1);
-    const bool act = gl < A.Wb;
     const unsigned gmask = group_mask(G);
     const int64_t groups_total = (int64_t)gridDim.x * (BD / G);
     const int64_t group_id = (int64_t)blockIdx.x * (BD / G) + tid / G;
     const unsigned nblocks = gridDim.x + A.bar_extra;
 
     const int64_t tree0 = *A.tree0;
-    for (int i = tid; i < A.Wb * 64; i += BD)
-        akey[KSLOT(i >> 6, i & 63)] = (uint32_t)sb_tree_key(A.S, tree0 + 64 * (int64_t)A.w0 + i);
+    for (int i = tid; i < A.H * 32; i += BD) {
+        const int64_t slot = 32 * (int64_t)A.h0 + i;
+        akey[KSLOT(i >> 5, i & 31)] = (uint32_t)sb_tree_key(A.S, tree0 + (A.perm ? (int64_t)A.perm[slot] : slot));
+    }
     if (tid == 0) s_any = 0;
     __syncthreads();
 
-    const int Wb = A.Wb, Wt = A.Wt, w0 = A.w0;
-    const int wofs = w0 + gl;
-    uint16_t* queue = queues + (tid / G) * (A.qcap * G);
+    // this lane's trees within its half-word
+    const int sub = gl & ((1 << A.ls) - 1), tpl = 32 >> A.ls;
+    const uint32_t mine = A.ls ? ((1u << tpl) - 1u) << (sub * tpl) : ~0u;
+    uint16_t* queue = queues + (tid / G) * (BFS_QUEUE * G);
     uint32_t* hxs = hx_tab + (tid / G) * 8;
+    const int ss = A.slices - 1;  // 1 or 2 slices
+    const int64_t units = A.n_items << ss;
     uint32_t n_scan = 0, n_hash = 0, n_hash_hub = 0;  // work counters
     // level 1 is built top-down before the launch (k_bfs_level1): every
     // neighbour of a root has that root as its only candidate
     int L = 2;
     while (true) {
-        const uint64_t* cur = (L & 1) ? A.fr0 : A.fr1;
-        uint64_t* nxt = (L & 1) ? A.fr1 : A.fr0;
+        const uint32_t* cur = (L & 1) ? A.fr0 : A.fr1;
+        uint32_t* nxt = (L & 1) ? A.fr1 : A.fr0;
         bool any_new = false;
 
         // ---- phase A: every work item (whole rows, and chunks of split rows)
-        // The items are sorted by descending degree and dealt out in rounds of
-        // one item per group, the order of the groups reversing every round,
-        // so that every group's sum of item sizes comes out about the same.
-        for (int64_t r = 0;; r++) {
-            const int64_t it_beg = r * groups_total + ((r & 1) ? groups_total - 1 - group_id : group_id);
-            if (r * groups_total >= A.n_items) break;
-            const int64_t it_end = min(A.n_items, it_beg + 1);
-            for (int64_t it = it_beg; it < it_end; it++) {
-                const sb_bfs_item itm = A.items[it];
-                const int32_t v = itm.v;
-                const int32_t d = A.done[v];
-                if (d >= 0 && L >= d + 3) continue;
-                const uint64_t vis_w = act ? A.vis[(int64_t)v * Wb + gl] : ~0ull;
-                const uint64_t U = ~vis_w;
-                const int32_t* cp = A.col + itm.beg;
-                const int len = itm.end - itm.beg;
-                const bool hub = itm.hub >= 0;
-                uint64_t once = 0, labx = 0;
-                // the pass below synchronises the group's lanes, so every lane of
-                // the group enters it (a lane with nothing to do has mask 0)
-                if (__any_sync(gmask, U != 0)) {
-                    const uint32_t goff = A.vgoff ? (uint32_t)A.vgoff[v] : 0u;
-                    const uint32_t y = sb_child_salt(A.S, (uint32_t)v - goff);
-                    if (U) n_scan += (uint32_t)len;
-                    // one pass: every candidate of every open tree is hashed (a
-                    // first pass that singled out the trees with two or more
-                    // candidates cost more than the few hashes it saved)
-                    best_reset<BD>(best, tid, U);
-                    uint32_t lbv[2] = {0u, 0u};
-                    scan_row<PAR, BD, G>(cp, len, cur, A.lab, Wb, Wt, wofs, gl, U, y, goff, akey, best, lbits, lbv,
-                                         bestu, queue, A.qcap, hxs, tid, gmask, once, hub ? n_hash_hub : n_hash);
-                    labx = (((uint64_t)lbv[1] << 32) | lbv[0]) & once;
-                }
-                if (hub) {
-                    // chunk of a split row: publish the chunk minima, one atomic per tree
-                    if (once) {
-                        uint64_t* hb = A.hubbest + ((int64_t)itm.hub * Wb + gl) * 64;
-                        for (uint64_t b = once; b;) {
-                            const int t = __ffsll((long long)b) - 1;
-                            b &= b - 1;
-                            const unsigned long long key = ((unsigned long long)best[BSLOT(tid, t)] << 32) |
-                                                           (PAR ? ((unsigned long long)(uint32_t)bestu[BSLOT(tid, t)] << 1) : 0ull) |
-                                                           ((labx >> t) & 1ull);
-                            atomicMin((unsigned long long*)(hb + t), key);
-                        }
-                        atomicOr((unsigned long long*)(A.hubnew + (int64_t)itm.hub * Wb + gl), once);
-                    }
-                    continue;
-                }
-                if (PAR && A.parents) {
-                    for (uint64_t b = once; b;) {
-                        const int t = __ffsll((long long)b) - 1;
+        // (sorted by descending degree; see BFS_SINGLE_PCT for who takes which)
+        auto unit = [&](int64_t x) {
+            const int sl = (int)(x & ss);
+            const int4 q = __ldg((const int4*)(A.items + (x >> ss)));  // vertex, CSR range, split row or -1
+            const int32_t v = q.x;
+            const int64_t dslot = (int64_t)v * A.slices + sl;
+            const int32_t d = A.done[dslot];
+            if (d >= 0 && L >= d + 3) return;
+            const int h = 32 * sl + (gl >> A.ls);
+            const bool act = h < A.H;
+            const uint32_t vis_w = act ? A.vis[(int64_t)v * A.H + h] : ~0u;
+            const uint32_t U = ~vis_w & mine;
+            const int len = q.z - q.y;
+            const bool hub = q.w >= 0;
+            uint32_t once = 0, lbv = 0;
+            // the pass below synchronises the group's lanes, so every lane of
+            // the group enters it (a lane with nothing to do has mask 0)
+            const uint32_t open = __ballot_sync(gmask, U != 0);
+            if (open) {
+                const uint32_t goff = A.vgoff ? (uint32_t)A.vgoff[v] : 0u;
+                const uint32_t y = sb_child_salt(A.S, (uint32_t)v - goff);
+                // neighbour entries per 64-tree word: the first open lane of
+                // the word's lanes counts them
+                const unsigned wl = 2u << A.ls;  // lanes of a word
+                const unsigned first = (unsigned)(tid & 31) & ~(wl - 1u);
+                if (U && (open & ((1u << (tid & 31)) - 1u) & ~((1u << first) - 1u)) == 0) n_scan += (uint32_t)len;
+                uint4* b4 = (uint4*)(best + BSLOT(tid, 0));
+#pragma unroll
+                for (int i = 0; i < 8; i++) b4[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+                // one pass: every candidate of every open tree is hashed
+                uint32_t& nh = hub ? n_hash_hub : n_hash;
+                const uint32_t* ak = akey + KSLOT(act ? h : 0, 0);
+                if constexpr (G == 32)
+                    scan_row_warp<PAR>(A.col + q.y, len, cur + h, A.lab + A.h0 + h, A.H, A.Ht, U, y, goff, ak,
+                                       best + BSLOT(tid, 0), lbv, PAR ? bestu + BSLOT(tid, 0) : nullptr, once, nh);
+                else
+                    scan_row<PAR, G>(A.col + q.y, len, cur + h, A.lab + A.h0 + h, A.H, A.Ht, gl, A.ls, U, y, goff,
+                                     akey + KSLOT(32 * sl, 0), ak, best, lbits, lbv, bestu, queue, hxs, tid, gmask, once,
+                                     nh);
+                lbv &= once;
+            }
+            if (hub) {
+                // chunk of a split row: publish the chunk minima, one atomic per tree
+                if (once) {
+                    uint64_t* hb = A.hubbest + ((int64_t)q.w * A.H + h) * 32;
+                    for (uint32_t b = once; b;) {
+                        const int t = __ffs((int)b) - 1;
                         b &= b - 1;
-                        A.parents[(64 * (int64_t)wofs + t) * A.n + v] = bestu[BSLOT(tid, t)];
+                        const unsigned long long key = ((unsigned long long)best[BSLOT(tid, t)] << 32) |
+                                                       (PAR ? ((unsigned long long)(uint32_t)bestu[BSLOT(tid, t)] << 1) : 0ull) |
+                                                       ((lbv >> t) & 1u);
+                        atomicMin((unsigned long long*)(hb + t), key);
                     }
+                    atomicOr(A.hubnew + (int64_t)q.w * A.H + h, once);
                 }
-                if (act) {
-                    if (once) {
-                        A.lab[(int64_t)v * Wt + wofs] |= labx & once;
-                        A.vis[(int64_t)v * Wb + gl] = vis_w | once;
-                        any_new = true;
-                    }
-                    nxt[(int64_t)v * Wb + gl] = once;
-                }
-                if (d < 0) {
-                    const bool full = (vis_w | once) == ~0ull;
-                    const bool all = __all_sync(gmask, full);
-                    if (all && gl == 0) A.done[v] = L;
+                return;
+            }
+            if (PAR && A.parents) {
+                for (uint32_t b = once; b;) {
+                    const int t = __ffs((int)b) - 1;
+                    b &= b - 1;
+                    const int64_t slot = 32 * (int64_t)(A.h0 + h) + t;
+                    A.parents[(A.perm ? (int64_t)A.perm[slot] : slot) * A.n + v] = bestu[BSLOT(tid, t)];
                 }
             }
-        }  // rounds
+            // the lanes of one half-word put their trees together
+            for (int s = 1; s < (1 << A.ls); s <<= 1) {
+                once |= __shfl_xor_sync(gmask, once, s);
+                lbv |= __shfl_xor_sync(gmask, lbv, s);
+            }
+            if (act && sub == 0) {
+                if (once) {
+                    if (lbv) A.lab[(int64_t)v * A.Ht + A.h0 + h] |= lbv;
+                    A.vis[(int64_t)v * A.H + h] = vis_w | once;
+                    any_new = true;
+                }
+                nxt[(int64_t)v * A.H + h] = once;
+            }
+            if (d < 0) {
+                const bool all = __all_sync(gmask, (vis_w | once) == ~0u);
+                if (all && gl == 0) A.done[dslot] = L;
+            }
+        };
+        const int64_t fixed = A.fixed_rounds;
+        for (int64_t r = 0; r < fixed; r++) {
+            const int64_t x = r * groups_total + ((r & 1) ? groups_total - 1 - group_id : group_id);
+            if (x < units) unit(x);
+        }
+        if (fixed * groups_total < units) {
+            constexpr int GW = 32 / G;  // groups of a warp
+            const int64_t first = fixed * groups_total, singles = A.single_tickets;
+            uint32_t* ctr = A.sync + 36 + L % 3;
+            auto ticket = [&]() { return (tid & 31) == 0 ? atomicAdd(ctr, 1u) : 0u; };
+            unsigned nt = ticket();  // always one ahead
+            while (true) {
+                const int64_t t = __shfl_sync(0xffffffffu, nt, 0);
+                const int64_t b = first + (t < singles ? t : singles + (t - singles) * A.grab) * GW;
+                if (b >= units) break;
+                nt = ticket();
+                const int cnt = t < singles ? 1 : A.grab;
+                for (int i = 0; i < cnt; i++) {
+                    const int64_t x = b + i * GW + (tid & 31) / G;
+                    if (x < units) unit(x);
+                }
+            }
+        }
 
-        // ---- phase B: resolve split rows
+        // ---- phase B: resolve split rows, a warp each
         if (A.n_hubs > 0) {
             grid_barrier(A.sync, nblocks, A.wait);
-            for (int64_t h = group_id; h < A.n_hubs; h += groups_total) {
-                const int32_t v = A.hub_vertex[h];
-                const int32_t d = A.done[v];
-                if (d >= 0 && L >= d + 3) continue;
-                uint64_t nw = 0, vis_w = ~0ull;
-                if (act) {
-                    vis_w = A.vis[(int64_t)v * Wb + gl];
-                    uint64_t* hn = A.hubnew + h * Wb + gl;
-                    nw = *hn & ~vis_w;
-                    *hn = 0;
-                    uint64_t labx = 0;
-                    uint64_t* hb = A.hubbest + (h * Wb + gl) * 64;
-                    for (uint64_t b = nw; b;) {
-                        const int t = __ffsll((long long)b) - 1;
-                        b &= b - 1;
-                        const uint64_t key = hb[t];
-                        hb[t] = ~0ull;
-                        labx |= (key & 1ull) << t;
-                        if (PAR && A.parents)
-                            A.parents[(64 * (int64_t)wofs + t) * A.n + v] = (int32_t)((key >> 1) & SB_ID_MASK);
-                    }
-                    if (nw) {
-                        A.lab[(int64_t)v * Wt + wofs] |= labx;
-                        A.vis[(int64_t)v * Wb + gl] = vis_w | nw;
-                        any_new = true;
-                    }
-                    nxt[(int64_t)v * Wb + gl] = nw;
-                }
-                if (d < 0) {
-                    const bool all = __all_sync(gmask, (vis_w | nw) == ~0ull);
-                    if (all && gl == 0) A.done[v] = L;
-                }
-            }
+            for (int64_t x = (int64_t)blockIdx.x * (BD / 32) + tid / 32; x < (A.n_hubs << ss);
+                 x += (int64_t)gridDim.x * (BD / 32))
+                any_new |= bfs_hub<PAR>(A, L, nxt, x >> ss, (int)(x & ss));
         }
 
         // ---- end of level: any tree grew?
@@ -505,7 +551,10 @@ __global__ void __launch_bounds__(PAR ? BFS_THREADS_PAR : BFS_THREADS, PAR ? 2 :
         if (tid == 0) {
             if (s_any) atomicOr(A.sync + (L % 3), 1u);
             s_any = 0;
-            if (blockIdx.x == 0) A.sync[(L + 1) % 3] = 0;
+            if (blockIdx.x == 0) {
+                A.sync[(L + 1) % 3] = 0;
+                A.sync[36 + (L + 1) % 3] = 0;
+            }
         }
         grid_barrier(A.sync, nblocks, A.wait);
         // one reader per block, so that every thread of a block leaves the
@@ -547,10 +596,11 @@ __global__ void __launch_bounds__(PAR ? BFS_THREADS_PAR : BFS_THREADS, PAR ? 2 :
 // first read.  The error word sync[6] is cleared per batch, so that an error
 // of an earlier launch stays.)
 __global__ void k_bfs_init(int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_t* vis, uint64_t* fr1, uint64_t* lab,
-                           int32_t* done, int64_t nh, uint64_t* hubnew, uint64_t* hubbest, uint32_t* sync)
+                           int32_t* done, int slices, int64_t nh, uint64_t* hubnew, uint64_t* hubbest, uint32_t* sync)
 {
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     if (i0 < 6) sync[i0] = 0;
+    if (i0 >= 36 && i0 < 39) sync[i0] = 0;
     const int64_t total = n * Wb;
     for (int64_t i = i0; i < total; i += step) {
         int64_t v = i / Wb;
@@ -560,7 +610,7 @@ __global__ void k_bfs_init(int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_
         vis[i] = ~active;
         fr1[i] = 0;
         lab[v * Wt + w0 + w] = 0;
-        if (w == 0) done[v] = -1;
+        if (w < slices) done[v * slices + w] = -1;
     }
     for (int64_t i = i0; i < nh * Wb * 64; i += step) {
         hubbest[i] = ~0ull;
@@ -574,7 +624,7 @@ __global__ void k_bfs_init(int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_
 // tree of the launch); trees of one word may reach the same vertex, hence
 // the atomics.  Frontier of level 1 -> fr1 (read as the current frontier of
 // level 2).
-__global__ void k_bfs_level1(int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_t S, const int64_t* tree0p,
+__global__ void k_bfs_level1(const int32_t* perm, int64_t n, int Wb, int Wt, int w0, int64_t K, uint64_t S, const int64_t* tree0p,
                              const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, uint64_t* vis,
                              uint64_t* fr1, uint64_t* lab, int32_t* parents, const int32_t* voff, int64_t G)
 {
@@ -584,8 +634,8 @@ __global__ void k_bfs_level1(int64_t n, int Wb, int Wt, int w0, int64_t K, uint6
     if (warp >= per * G) return;
     const int64_t g = warp / per;
     const int64_t i = warp - g * per;         // tree within this launch
-    const int64_t tb = 64 * (int64_t)w0 + i;  // tree within the batch
-    if (tb >= K) return;
+    if (64 * (int64_t)w0 + i >= K) return;
+    const int64_t tb = perm ? perm[64 * w0 + i] : 64 * (int64_t)w0 + i;
     const uint64_t key = sb_tree_key(S, *tree0p + tb);
     const int64_t base = voff ? voff[g] : 0;
     const int64_t ng = voff ? voff[g + 1] - voff[g] : n;
@@ -728,15 +778,16 @@ __global__ void __launch_bounds__(HT_THREADS, 4) k_state_hash_tab(const uint64_t
 }
 
 // canonical flip of the raw sums: trees whose vertex 0 (of the tree's graph)
-// is labelled 1 take the complement's weight
-__global__ void k_state_hash_flip(unsigned long long* H, const unsigned long long* wsum, const uint64_t* flipw, int W,
-                                  int64_t KP, int64_t G)
+// is labelled 1 take the complement's weight.  Slot order in, tree order out.
+__global__ void k_state_hash_flip(const unsigned long long* Hraw, unsigned long long* H, const unsigned long long* wsum,
+                                  const uint64_t* flipw, const int32_t* perm, int W, int64_t KP, int64_t G)
 {
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= KP * G) return;
     const int64_t g = x / KP;
     const int64_t t = x - g * KP;
-    if ((flipw[g * W + t / 64] >> (t % 64)) & 1ull) H[x] = wsum[g] - H[x];
+    const unsigned long long h = Hraw[x];
+    H[g * KP + (perm ? (int64_t)perm[t] : t)] = ((flipw[g * W + t / 64] >> (t % 64)) & 1ull) ? wsum[g] - h : h;
 }
 
 __global__ void k_canon_out(const uint64_t* __restrict__ lab, int64_t total, int W, int64_t K,
@@ -753,19 +804,48 @@ __global__ void k_canon_out(const uint64_t* __restrict__ lab, int64_t total, int
     }
 }
 
-// --------------------------------------------------------------- host side
-static int group_for(int Wb)
+// The same for slots in another order than the trees (one graph).  A block
+// stages the canonical rows of 32 vertices; a warp takes an output half-word
+// at a time, whose 32 slots its lanes keep while they pick their bit of every
+// vertex.
+#define CO_THREADS 256
+#define CO_ROWS 32
+__global__ void __launch_bounds__(CO_THREADS) k_canon_out_order(const uint32_t* __restrict__ lab, int64_t n, int Ht,
+                                                                int64_t K, const uint32_t* __restrict__ flip,
+                                                                const int32_t* __restrict__ slot,
+                                                                uint32_t* __restrict__ out)
 {
-    int g = 1;
-    while (g < Wb) g <<= 1;
-    return g;
+    extern __shared__ uint32_t co[];
+    uint32_t* rows = co;                   // CO_ROWS x Ht canonical rows, slot order
+    uint32_t* res = co + CO_ROWS * Ht;     // the same, tree order
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t v0 = (int64_t)blockIdx.x * CO_ROWS; v0 < n; v0 += (int64_t)gridDim.x * CO_ROWS) {
+        const int words = (int)min((int64_t)CO_ROWS, n - v0) * Ht;
+        for (int i = threadIdx.x; i < words; i += CO_THREADS) rows[i] = lab[v0 * Ht + i] ^ flip[i % Ht];
+        __syncthreads();
+        for (int h = warp; h < Ht; h += CO_THREADS / 32) {
+            const int s = slot[32 * h + lane];
+            const uint32_t bit = 32 * (int64_t)h + lane < K ? 1u << (s & 31) : 0u;
+            const uint32_t* src = rows + (s >> 5);
+            uint32_t keep = 0;
+#pragma unroll
+            for (int r = 0; r < CO_ROWS; r++) {  // rows past n are read as they are and not written
+                const uint32_t b = __ballot_sync(0xffffffffu, src[r * Ht] & bit);
+                if (lane == r) keep = b;
+            }
+            res[lane * Ht + h] = keep;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < words; i += CO_THREADS) out[v0 * Ht + i] = res[i];
+        __syncthreads();
+    }
 }
 
+// --------------------------------------------------------------- host side
 template <bool PAR>
 static const void* bfs_kernel(int G)
 {
     switch (G) {
-    case 1: return (const void*)k_bfs<1, PAR>;
     case 2: return (const void*)k_bfs<2, PAR>;
     case 4: return (const void*)k_bfs<4, PAR>;
     case 8: return (const void*)k_bfs<8, PAR>;
@@ -787,43 +867,47 @@ static sb_status ensure_sync(sb_ctx* c)
 static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
 {
     const bool par = parents != nullptr;
-    // lanes beyond the launch's words still share the hash rounds
-    const int Gw = group_for(Wb), Gt = (int)c->tune[SB_TUNE_BFS_GROUP];
-    const int G = (Gt > Gw && Gt <= 2 * Gw) ? Gt : Gw;  // widened at most twofold
     const int BD = par ? BFS_THREADS_PAR : BFS_THREADS;
-    const void* fn = par ? bfs_kernel<true>(G) : bfs_kernel<false>(G);
-    // shared memory of a block with q queue entries per lane; the largest q that
-    // keeps the most blocks resident
-    auto smem_for = [&](int q) -> size_t {
-        return sizeof(uint32_t) * ((size_t)Wb * 65 + 65 * BD + 2 * BD) + sizeof(uint16_t) * (size_t)((q * BD + 1) & ~1) +
-               (par ? sizeof(int32_t) * 65 * BD : 0) + sizeof(uint32_t) * 8 * (BD / G);
-    };
-    SB_CHECK_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_for(BFS_QUEUE_MAX)));
-    int per_sm = 0, qcap = BFS_QUEUE_MAX;
-    for (int q = BFS_QUEUE_MAX; q >= BFS_QUEUE_MIN; q--) {
-        int b = 0;
-        SB_CHECK_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, BD, smem_for(q)));
-        if (b > per_sm) {
-            per_sm = b;
-            qcap = q;
-        }
+    const int H = 2 * Wb, slices = H > 32 ? 2 : 1;
+    int G = 2;  // lanes of a vertex: one per half-word
+    while (G < H && G < 32) G <<= 1;
+    // A graph too small to fill the SMs that way spreads the trees of a
+    // half-word over more lanes, which shortens every lane's run of hashes
+    // (1000 vertices, 64 trees: 70 us with 2 lanes per vertex, 43 with 32).  The
+    // knob asks for that width.
+    int ls = 0;
+    const int Gt = (int)c->tune[SB_TUNE_BFS_GROUP];
+    while (G < Gt) {
+        G <<= 1;
+        ls++;
     }
-    const size_t smem = smem_for(qcap);
+    while (Gt == 0 && G < 32 && c->n_items * slices * G < (int64_t)c->num_sms * BFS_SPREAD_THREADS) {
+        G <<= 1;
+        ls++;
+    }
+    const void* fn = par ? bfs_kernel<true>(G) : bfs_kernel<false>(G);
+    const size_t smem = sizeof(uint32_t) * ((size_t)BSLOT(BD, 0) * (par ? 2 : 1) + (size_t)H * 33 + BD + 8 * (BD / G)) +
+                        sizeof(uint16_t) * BFS_QUEUE * BD;
+    SB_CHECK_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    SB_CHECK_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, BD, smem));
     if (per_sm < 1) return sb_fail(c, SB_ERR_CUDA, "BFS kernel does not fit on an SM");
-    // one group per work item at most: every further block would only lengthen
-    // the grid barriers (1000 vertices, one word: 8 blocks instead of 760)
+    // one group per work unit at most: every further block would only lengthen
+    // the grid barriers (1000 vertices, one word: 105 us with 8 blocks, 120
+    // with 760, one lane per word)
     unsigned nblocks = (unsigned)std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)per_sm * c->num_sms, sb_cdiv(c->n_items, BD / G)));
+        1, std::min<int64_t>((int64_t)per_sm * c->num_sms, sb_cdiv(c->n_items * slices, BD / G)));
     const int64_t n = c->n;
     const int64_t ngraphs = c->batch_G > 0 ? c->batch_G : 1;
+    const int32_t* perm = c->ordered ? c->order : nullptr;
     unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(std::max(n, c->n_hubs * 64) * Wb, 256), (int64_t)c->num_sms * 16);
-    k_bfs_init<<<g, 256, 0, c->stream>>>(n, Wb, c->W, w0, c->K, c->vis, c->fr1, c->labels, c->done, c->n_hubs,
+    k_bfs_init<<<g, 256, 0, c->stream>>>(n, Wb, c->W, w0, c->K, c->vis, c->fr1, c->labels, c->done, slices, c->n_hubs,
                                          c->hubnew, c->hubbest, c->sync);
     SB_TRY(sb_after_launch(c, "k_bfs_init"));
     {
         const int64_t warps = 64 * (int64_t)Wb * ngraphs;
         k_bfs_level1<<<(unsigned)sb_cdiv(warps * 32, 256), 256, 0, c->stream>>>(
-            n, Wb, c->W, w0, c->K, sb_seed_key(c->seed), sb_tree0_ptr(c->sync), c->rowptr, c->col, c->vis, c->fr1,
+            perm, n, Wb, c->W, w0, c->K, sb_seed_key(c->seed), sb_tree0_ptr(c->sync), c->rowptr, c->col, c->vis, c->fr1,
             c->labels, parents, c->batch_G > 0 ? c->b_voff : nullptr, ngraphs);
         SB_TRY(sb_after_launch(c, "k_bfs_level1"));
     }
@@ -833,25 +917,33 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
     A.col = c->col;
     A.hub_vertex = c->hub_vertex;
     A.n_hubs = c->n_hubs;
-    A.lab = c->labels;
-    A.Wt = c->W;
-    A.w0 = w0;
-    A.Wb = Wb;
-    A.vis = c->vis;
-    A.fr0 = c->fr0;
-    A.fr1 = c->fr1;
+    A.lab = (uint32_t*)c->labels;
+    A.Ht = 2 * c->W;
+    A.h0 = 2 * w0;
+    A.H = H;
+    A.slices = slices;
+    A.ls = ls;
+    {
+        const int64_t units = c->n_items * slices, groups = (int64_t)nblocks * (BD / G), rounds = units / groups;
+        A.fixed_rounds = G == 32 ? 1 : std::max<int64_t>(1, rounds * BFS_FIXED_PCT / 100);
+        A.single_tickets = G == 32 ? units * BFS_SINGLE_PCT / 100 : 0;
+        A.grab = G == 32 && rounds >= 1000 ? 8 : 4;
+    }
+    A.vis = (uint32_t*)c->vis;
+    A.fr0 = (uint32_t*)c->fr0;
+    A.fr1 = (uint32_t*)c->fr1;
     A.done = c->done;
-    A.hubnew = c->hubnew;
+    A.hubnew = (uint32_t*)c->hubnew;
     A.hubbest = c->hubbest;
     A.sync = c->sync;
     A.parents = parents;
     A.n = n;
     A.S = sb_seed_key(c->seed);
     A.tree0 = sb_tree0_ptr(c->sync);
+    A.perm = perm;
     A.vgoff = c->batch_G > 0 ? c->vgoff : nullptr;
     A.wait = sb_wait_cycles(c);
     A.bar_extra = c->tune[SB_TUNE_STALL_TEST] ? 1u : 0u;
-    A.qcap = qcap;
     void* args[] = {&A};
     {
         // a cooperative launch (every block resident for the grid barrier),
@@ -870,6 +962,56 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
         SbProf prof(c, SB_PROF_BFS);
         SB_CHECK_CUDA(c, cudaLaunchKernelExC(&cfg, fn, args));
         return sb_after_launch(c, "k_bfs");
+    }
+}
+
+// Expected depth of every tree of a single-graph batch, as the number of
+// entries in the rows of its root's neighbours (most entries first: such a
+// root reaches the bulk of the graph one level earlier).  One block per tree.
+#define ORD_THREADS 128
+__global__ void __launch_bounds__(ORD_THREADS) k_tree_keys(int64_t n, int64_t K, uint64_t S, const int64_t* tree0p,
+                                                           const int32_t* __restrict__ rowptr,
+                                                           const int32_t* __restrict__ col, uint64_t* __restrict__ keys)
+{
+    const int64_t t = blockIdx.x;
+    const int64_t r = sb_root(sb_tree_key(S, *tree0p + t), n);
+    unsigned sum = 0;  // at most 2 m < 2^31
+    for (int32_t j = rowptr[r] + (int)threadIdx.x; j < rowptr[r + 1]; j += ORD_THREADS) {
+        const int64_t u = (uint32_t)col[j] & SB_ID_MASK;
+        sum += (unsigned)(rowptr[u + 1] - rowptr[u]);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    __shared__ unsigned part[ORD_THREADS / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < ORD_THREADS / 32; i++) sum += part[i];
+        keys[t] = ((uint64_t)(~sum) << 32) | (uint64_t)t;
+    }
+}
+
+// order[slot] = tree, order[slots + tree] = slot.  The trees by ascending key
+// (a tree's rank is the number of smaller keys, which are distinct; one warp
+// counts them) are dealt out over the full half-words, so that each holds the
+// same mix of depths: the lanes of a group then have about as many candidates
+// each.  The last K % 32 trees and the slots past K come after them.
+__global__ void __launch_bounds__(ORD_THREADS) k_tree_order(const uint64_t* __restrict__ keys, int64_t K, int64_t slots,
+                                                            int32_t* __restrict__ order)
+{
+    const int64_t t = ((int64_t)blockIdx.x * ORD_THREADS + threadIdx.x) >> 5;
+    if (t >= slots) return;
+    unsigned rank = (unsigned)t;
+    if (t < K) {
+        const uint64_t key = keys[t];
+        rank = 0;
+        for (int64_t i = threadIdx.x & 31; i < K; i += 32) rank += keys[i] < key ? 1u : 0u;
+        rank = __reduce_add_sync(0xffffffffu, rank);
+        const unsigned full = (unsigned)(K >> 5);
+        if (rank < 32 * full) rank = 32 * (rank % full) + rank / full;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        order[rank] = (int32_t)t;
+        order[slots + t] = (int32_t)rank;
     }
 }
 
@@ -938,7 +1080,9 @@ sb_status sb_batch_begin(sb_ctx* c, uint64_t seed, int64_t tree_begin, int64_t K
     // kept while large enough, so that repeated calls allocate nothing
     sb_status st = sb_ensure(c, (void**)&c->flipw, &c->flipw_cap, sizeof(uint64_t) * W * G);
     if (st == SB_OK) st = sb_ensure(c, (void**)&c->hashes, &c->hashes_cap, sizeof(uint64_t) * 64 * W * G);
+    if (st == SB_OK) st = sb_ensure(c, (void**)&c->hraw, &c->hraw_cap, sizeof(uint64_t) * 64 * W * G);
     if (st == SB_OK) st = sb_ensure(c, (void**)&c->counts, &c->counts_cap, sizeof(int32_t) * 64 * W * G);
+    c->ordered = false;
     c->has_batch = false;
     if (st != SB_OK || !c->labels || !c->flipw || !c->hashes || !c->counts)
         return sb_fail(c, SB_ERR_OOM, "batch storage (n=%lld, K=%lld)", (long long)n, (long long)K);
@@ -958,7 +1102,7 @@ sb_status sb_batch_end(sb_ctx* c)
     const int W = c->W;
     SB_TRY(sb_ensure(c, (void**)&c->hwsum, &c->hwsum_cap, sizeof(uint64_t) * (size_t)G));
     k_flip<<<(unsigned)sb_cdiv(64 * (int64_t)W * G, 256), 256, 0, c->stream>>>(
-        c->labels, W, c->flipw, c->batch_G > 0 ? c->b_voff : nullptr, G, (unsigned long long*)c->hashes,
+        c->labels, W, c->flipw, c->batch_G > 0 ? c->b_voff : nullptr, G, (unsigned long long*)c->hraw,
         (unsigned long long*)c->hwsum);
     SB_TRY(sb_after_launch(c, "k_flip"));
     {
@@ -968,10 +1112,11 @@ sb_status sb_batch_end(sb_ctx* c)
         const int64_t per = sb_cdiv(ngroups, nblk);
         k_state_hash_tab<<<(unsigned)sb_cdiv(ngroups, per), HT_THREADS, 0, c->stream>>>(
             c->labels, n, W, c->vweight, c->batch_G > 0 ? c->vgid : nullptr, 64 * (int64_t)W, per,
-            (unsigned long long*)c->hashes, (unsigned long long*)c->hwsum);
+            (unsigned long long*)c->hraw, (unsigned long long*)c->hwsum);
         SB_TRY(sb_after_launch(c, "k_state_hash_tab"));
         k_state_hash_flip<<<(unsigned)sb_cdiv(64 * (int64_t)W * G, 256), 256, 0, c->stream>>>(
-            (unsigned long long*)c->hashes, (const unsigned long long*)c->hwsum, c->flipw, W, 64 * (int64_t)W, G);
+            (const unsigned long long*)c->hraw, (unsigned long long*)c->hashes, (const unsigned long long*)c->hwsum,
+            c->flipw, c->ordered ? c->order : nullptr, W, 64 * (int64_t)W, G);
         SB_TRY(sb_after_launch(c, "k_state_hash_flip"));
     }
     c->has_batch = true;
@@ -1000,14 +1145,31 @@ static sb_status bfs_alloc(sb_ctx* c)
         c->vis = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * words);
         c->fr0 = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * words);
         c->fr1 = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * words);
-        c->hubnew = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * (size_t)(c->n_hubs > 0 ? c->n_hubs : 1) * Wb_max);
-        c->hubbest =
-            (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * (size_t)(c->n_hubs > 0 ? c->n_hubs : 1) * Wb_max * 64);
+        const size_t hw = (size_t)(c->n_hubs > 0 ? c->n_hubs : 1) * Wb_max;
+        c->hubnew = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * hw);
+        c->hubbest = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * hw * 64);
         c->bfs_cap_words = (c->vis && c->fr0 && c->fr1 && c->hubnew && c->hubbest) ? words : 0;
     }
-    if (!c->done) c->done = (int32_t*)sb_dalloc(c, sizeof(int32_t) * (size_t)n);
+    if (!c->done) c->done = (int32_t*)sb_dalloc(c, sizeof(int32_t) * 2 * (size_t)n);  // two slices at most
     if (!c->bfs_cap_words || !c->done)
         return sb_fail(c, SB_ERR_OOM, "BFS batch storage (n=%lld, K=%lld)", (long long)n, (long long)c->K);
+    return SB_OK;
+}
+
+// Fills the slots by the trees' expected depth (see BFS_ORDER_MIN).
+static sb_status bfs_order(sb_ctx* c)
+{
+    if (c->batch_G > 0 || c->K <= 32 || c->n < BFS_ORDER_MIN) return SB_OK;
+    const int64_t slots = 64 * (int64_t)c->W;
+    SB_TRY(sb_ensure(c, (void**)&c->order, &c->order_cap, sizeof(int32_t) * 2 * (size_t)slots));
+    SB_TRY(sb_ensure(c, (void**)&c->order_keys, &c->order_keys_cap, sizeof(uint64_t) * (size_t)slots));
+    k_tree_keys<<<(unsigned)c->K, ORD_THREADS, 0, c->stream>>>(c->n, c->K, sb_seed_key(c->seed), sb_tree0_ptr(c->sync),
+                                                               c->rowptr, c->col, c->order_keys);
+    SB_TRY(sb_after_launch(c, "k_tree_keys"));
+    k_tree_order<<<(unsigned)sb_cdiv(slots * 32, ORD_THREADS), ORD_THREADS, 0, c->stream>>>(c->order_keys, c->K, slots,
+                                                                                          c->order);
+    SB_TRY(sb_after_launch(c, "k_tree_order"));
+    c->ordered = true;
     return SB_OK;
 }
 
@@ -1033,6 +1195,7 @@ extern "C" sb_status sb_sample_trees(sb_ctx* c, uint64_t seed, int64_t tree_begi
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
     SB_TRY(sb_batch_begin(c, seed, tree_begin, K));
     SB_TRY(bfs_alloc(c));
+    SB_TRY(bfs_order(c));
     const sb_status st = bfs_enqueue(c, parents_out);
     c->tune[SB_TUNE_STALL_TEST] = 0;  // a test of the timeout path covers one call
     SB_TRY(st);
@@ -1193,9 +1356,18 @@ extern "C" sb_status sb_label(sb_ctx* c, uint64_t* labels_out)
     size_t bytes = sizeof(uint64_t) * (size_t)total;
     uint64_t* tmp = (uint64_t*)sb_dalloc(c, bytes);
     if (!tmp) return sb_fail(c, SB_ERR_OOM, "label export");
-    unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(total, 256), (int64_t)c->num_sms * 16);
-    k_canon_out<<<g, 256, 0, c->stream>>>(c->labels, total, c->W, c->K, c->flipw,
-                                          c->batch_G > 0 ? c->vgid : nullptr, tmp);
+    if (c->ordered) {
+        const int Ht = 2 * c->W;
+        const size_t smem = sizeof(uint32_t) * 2 * CO_ROWS * (size_t)Ht;  // at most 32 KB
+        const unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(c->n, CO_ROWS), (int64_t)c->num_sms * 8);
+        k_canon_out_order<<<g, CO_THREADS, smem, c->stream>>>((const uint32_t*)c->labels, c->n, Ht, c->K,
+                                                              (const uint32_t*)c->flipw, c->order + 32 * Ht,
+                                                              (uint32_t*)tmp);
+    } else {
+        unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(total, 256), (int64_t)c->num_sms * 16);
+        k_canon_out<<<g, 256, 0, c->stream>>>(c->labels, total, c->W, c->K, c->flipw,
+                                              c->batch_G > 0 ? c->vgid : nullptr, tmp);
+    }
     sb_status st = sb_after_launch(c, "k_canon_out");
     if (st == SB_OK) st = sb_copy_out(c, labels_out, tmp, bytes);
     cudaStreamSynchronize(c->stream);

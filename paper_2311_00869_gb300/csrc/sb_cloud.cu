@@ -321,7 +321,7 @@ __global__ void k_cloud_assign_scalable(const uint64_t* __restrict__ hashes, con
     meta[0] = ns;
 }
 
-// Canonical label bit of batch tree i at vertex v.
+// Canonical label bit of slot i at vertex v.
 __device__ __forceinline__ uint32_t cl_bit(const uint64_t* row, const uint64_t* flipw, int64_t i)
 {
     const int w = (int)(i >> 6), b = (int)(i & 63);
@@ -338,8 +338,8 @@ __device__ __forceinline__ uint32_t cl_bit(const uint64_t* row, const uint64_t* 
 #define CLV_THREADS 256
 __global__ void __launch_bounds__(CLV_THREADS)
     k_cloud_verify(const uint64_t* __restrict__ lab, int64_t n, int W, const uint64_t* __restrict__ flipw, int64_t K,
-                   const int32_t* __restrict__ assign, const int32_t* __restrict__ rep, uint64_t* bits,
-                   int64_t max_states, int32_t* mismatch)
+                   const int32_t* __restrict__ slot, const int32_t* __restrict__ assign,
+                   const int32_t* __restrict__ rep, uint64_t* bits, int64_t max_states, int32_t* mismatch)
 {
     extern __shared__ uint64_t rows[];  // 64 x W
     const int64_t chunk = blockIdx.x;
@@ -366,13 +366,15 @@ __global__ void __launch_bounds__(CLV_THREADS)
     for (int64_t i = threadIdx.x; i < K; i += CLV_THREADS) {
         const int32_t s = assign[i];
         if (s < 0) continue;
-        const uint64_t col = rows[(i & 63) * W + (i >> 6)];
+        const int si = slot ? slot[i] : (int)i;  // where tree i's labels are
+        const uint64_t col = rows[(si & 63) * W + (si >> 6)];
         const int32_t creator = rep[s];
-        uint64_t* slot = bits + chunk * max_states + s;
+        uint64_t* stored = bits + chunk * max_states + s;
         if (creator == (int32_t)i) {
-            *slot = col;
+            *stored = col;
         } else {
-            const uint64_t other = creator >= 0 ? rows[(creator & 63) * W + (creator >> 6)] : *slot;
+            const int sc = creator < 0 ? 0 : slot ? slot[creator] : creator;
+            const uint64_t other = creator >= 0 ? rows[(sc & 63) * W + (sc >> 6)] : *stored;
             if (other != col) mismatch[i] = 1;
         }
     }
@@ -380,8 +382,10 @@ __global__ void __launch_bounds__(CLV_THREADS)
 
 // Exact comparison (mode 0) or storage (mode 1) of one tree against one state.
 __global__ void k_cloud_pair(const uint64_t* __restrict__ lab, int64_t n, int W, const uint64_t* __restrict__ flipw,
-                             int64_t tree, int32_t state, uint64_t* bits, int64_t max_states, int mode, int32_t* differ)
+                             const int32_t* __restrict__ slot, int64_t tree, int32_t state, uint64_t* bits,
+                             int64_t max_states, int mode, int32_t* differ)
 {
+    if (slot) tree = slot[tree];
     const int64_t nchunks = sb_cdiv(n, 64);
     for (int64_t chunk = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; chunk < nchunks;
          chunk += (int64_t)gridDim.x * blockDim.x) {
@@ -389,9 +393,9 @@ __global__ void k_cloud_pair(const uint64_t* __restrict__ lab, int64_t n, int W,
         const int nv = (int)min((int64_t)64, n - v0);
         uint64_t col = 0;
         for (int r = 0; r < nv; r++) col |= (uint64_t)cl_bit(lab + (v0 + r) * W, flipw, tree) << r;
-        uint64_t* slot = bits + chunk * max_states + state;
-        if (mode == 1) *slot = col;
-        else if (*slot != col) atomicOr(differ, 1);
+        uint64_t* stored = bits + chunk * max_states + state;
+        if (mode == 1) *stored = col;
+        else if (*stored != col) atomicOr(differ, 1);
     }
 }
 
@@ -468,6 +472,7 @@ static sb_status cloud_resolve_collisions(sb_ctx* c)
     SB_CHECK_CUDA(c, cudaMemcpy(hashes.data(), c->hashes, sizeof(uint64_t) * K, cudaMemcpyDeviceToHost));
     SB_CHECK_CUDA(c, cudaMemcpy(counts.data(), c->counts, sizeof(int32_t) * K, cudaMemcpyDeviceToHost));
     int32_t* differ = c->cl_meta + 4;
+    const int32_t* slot = c->ordered ? c->order + 64 * (int64_t)c->W : nullptr;
     int32_t ns = meta[0];
     const int64_t nchunks = sb_cdiv(c->n, 64);
     unsigned g = (unsigned)std::min<int64_t>(sb_cdiv(nchunks, 256), (int64_t)c->num_sms * 8);
@@ -484,7 +489,7 @@ static sb_status cloud_resolve_collisions(sb_ctx* c)
                 if (entries[st].S == counts[i]) {
                     int32_t h_differ = 0;
                     SB_CHECK_CUDA(c, cudaMemsetAsync(differ, 0, sizeof(int32_t), c->stream));
-                    k_cloud_pair<<<g, 256, 0, c->stream>>>(c->labels, c->n, c->W, c->flipw, i, st, c->cl_bits,
+                    k_cloud_pair<<<g, 256, 0, c->stream>>>(c->labels, c->n, c->W, c->flipw, slot, i, st, c->cl_bits,
                                                           c->cl_max, 0, differ);
                     SB_TRY(sb_after_launch(c, "k_cloud_pair"));
                     SB_CHECK_CUDA(c, cudaMemcpyAsync(&h_differ, differ, sizeof(int32_t), cudaMemcpyDeviceToHost,
@@ -510,7 +515,7 @@ static sb_status cloud_resolve_collisions(sb_ctx* c)
             entries[ns].S = counts[i];
             entries[ns].count = 1;
             entries[ns].first_tree = c->tree_begin + i;
-            k_cloud_pair<<<g, 256, 0, c->stream>>>(c->labels, c->n, c->W, c->flipw, i, ns, c->cl_bits, c->cl_max, 1,
+            k_cloud_pair<<<g, 256, 0, c->stream>>>(c->labels, c->n, c->W, c->flipw, slot, i, ns, c->cl_bits, c->cl_max, 1,
                                                   differ);
             SB_TRY(sb_after_launch(c, "k_cloud_pair"));
             ns++;
@@ -561,7 +566,8 @@ sb_status sb_cloud_insert_batch(sb_ctx* c)
     size_t smem = sizeof(uint64_t) * 64 * (size_t)c->W;
     if (smem > 48 * 1024)
         SB_CHECK_CUDA(c, cudaFuncSetAttribute(k_cloud_verify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_cloud_verify<<<(unsigned)nchunks, CLV_THREADS, smem, c->stream>>>(c->labels, c->n, c->W, c->flipw, c->K,
+    const int32_t* slot = c->ordered ? c->order + 64 * (int64_t)c->W : nullptr;
+    k_cloud_verify<<<(unsigned)nchunks, CLV_THREADS, smem, c->stream>>>(c->labels, c->n, c->W, c->flipw, c->K, slot,
                                                                          c->cl_assign, c->cl_rep, c->cl_bits,
                                                                          c->cl_max, c->cl_mismatch);
     SB_TRY(sb_after_launch(c, "k_cloud_verify"));

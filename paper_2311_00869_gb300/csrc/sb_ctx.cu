@@ -190,6 +190,12 @@ void sb_release_batch(sb_ctx* c)
     c->flipw_cap = 0;
     SB_FREE(hashes);
     c->hashes_cap = 0;
+    SB_FREE(hraw);
+    c->hraw_cap = 0;
+    SB_FREE(order);
+    SB_FREE(order_keys);
+    c->order_cap = c->order_keys_cap = 0;
+    c->ordered = false;
     SB_FREE(hwsum);
     c->hwsum_cap = 0;
     SB_FREE(counts);

@@ -121,9 +121,16 @@ struct sb_ctx {
     uint64_t seed = 0;
     int64_t tree_begin = 0, K = 0;
     int W = 0;                    // words = ceil(K / 64)
-    uint64_t* labels = nullptr;   // n x W raw labels (root label 0)
+    uint64_t* labels = nullptr;   // n x W raw labels (root label 0), in slot order
     uint64_t* flipw = nullptr;    // W: label of vertex 0 per word (canonical flip)
     size_t flipw_cap = 0;
+    bool ordered = false;         // slots hold the trees in another order (else slot = tree)
+    int32_t* order = nullptr;     // [64 W] tree of each slot, then [64 W] slot of each tree
+    size_t order_cap = 0;
+    uint64_t* order_keys = nullptr;
+    size_t order_keys_cap = 0;
+    uint64_t* hraw = nullptr;     // per graph, 64 W: weight sums of the raw labels, in slot order
+    size_t hraw_cap = 0;
     uint64_t* hashes = nullptr;   // K
     size_t hashes_cap = 0;
     uint64_t* hwsum = nullptr;    // per graph: total vertex weight (state-hash complement)
@@ -144,7 +151,7 @@ struct sb_ctx {
     uint32_t* sync = nullptr;     // [0..2] level counters, [4] barrier count, [5] barrier gen, [6] error,
                                   // [16..27] work counters of the batch (sb_stats), [28] scorer error,
                                   // [32..33] first tree of the batch (int64, read by the kernels),
-                                  // [34] sticky errors of sb_batch_steps
+                                  // [34] sticky errors of sb_batch_steps, [36..38] BFS work tickets
     size_t bfs_cap_words = 0;
 
     // Kruskal (Boruvka) scratch, [vertex][tree of the pass]
@@ -313,9 +320,10 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, unsigned lane)
         const bool upper = (lane & (unsigned)s) == 0;
         // the upper row keeps its left columns and takes the partner's left
         // columns into its right ones; the lower row keeps its right columns
-        // and takes the partner's right columns into its left ones
+        // and takes the partner's right columns into its left ones (the bits
+        // that a rotation carries round fall in kept columns)
         const uint32_t keep = upper ? m : ~m;
-        const uint32_t t = upper ? (y << s) : (y >> s);
+        const uint32_t t = __funnelshift_l(y, y, upper ? s : 32 - s);
         x = (x & keep) | (t & ~keep);
     }
     return x;

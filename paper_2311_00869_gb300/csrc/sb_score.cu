@@ -32,6 +32,7 @@ struct ScoreArgs {
     const uint64_t* lab;  // n x Wt label words
     int Wt, w0, Wb;       // words [w0, w0 + Wb) of this launch, Wb <= 64
     const int32_t* vgid;  // graph of every vertex (batches of graphs) or null
+    const int32_t* perm;  // tree of each slot, or null (slot = tree)
     int64_t KP;           // count slots per graph
     uint32_t* counts;     // [graph * KP + 64 * word + bit]
     uint32_t* err;        // bit 0 set when a tile copy did not arrive in time
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(SC_THREADS, SEG ? 3 : 4) k_score(ScoreArgs A)
         acc.template flush_warp<G>(scnt + 64 * 32 * slice);
         __syncthreads();
         for (int i = tid; i < A.Wb * 64; i += SC_THREADS)
-            if (scnt[i]) atomicAdd(A.counts + 64 * A.w0 + i, scnt[i]);
+            if (scnt[i]) atomicAdd(A.counts + (A.perm ? A.perm[64 * A.w0 + i] : 64 * A.w0 + i), scnt[i]);
     }
 }
 
@@ -205,6 +206,7 @@ sb_status sb_score_enqueue(sb_ctx* c)
         A.w0 = 0;
         A.Wb = Wb;
         A.vgid = seg ? c->vgid : nullptr;
+        A.perm = c->ordered ? c->order : nullptr;
         A.KP = 64 * (int64_t)c->W;
         A.counts = (uint32_t*)c->counts;
         A.err = c->sync + 28;
