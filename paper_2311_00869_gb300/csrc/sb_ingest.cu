@@ -40,9 +40,11 @@ __global__ void k_validate(const int32_t* __restrict__ src, const int32_t* __res
 }
 
 // head flags of distinct pairs; flags[0] |= 1 on inconsistency, 2 on duplicate
+// (one atomic per block: duplicates are common)
 __global__ void k_heads(const uint64_t* __restrict__ keys, int64_t m, int32_t* __restrict__ head,
                         uint32_t* __restrict__ flags)
 {
+    uint32_t found = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         uint64_t k = keys[i];
         int h = 1;
@@ -50,11 +52,13 @@ __global__ void k_heads(const uint64_t* __restrict__ keys, int64_t m, int32_t* _
             uint64_t p = keys[i - 1];
             if ((p >> 1) == (k >> 1)) {
                 h = 0;
-                atomicOr(flags, (p & 1) != (k & 1) ? 1u : 2u);
+                found |= (p & 1) != (k & 1) ? 1u : 2u;
             }
         }
         head[i] = h;
     }
+    const uint32_t one = __syncthreads_or(found & 1u) ? 1u : 0u, two = __syncthreads_or(found & 2u) ? 2u : 0u;
+    if (threadIdx.x == 0 && (one | two)) atomicOr(flags, one | two);
 }
 
 __global__ void k_compact_keys(const uint64_t* __restrict__ keys, const int32_t* __restrict__ head,
@@ -65,6 +69,14 @@ __global__ void k_compact_keys(const uint64_t* __restrict__ keys, const int32_t*
 }
 
 // ------------------------------------------------------------- union-find
+// The edges come sorted, so that neighbouring threads hook the same vertices
+// and build long chains: sparse samples first, paths compressed in between,
+// and the full pass then finds most edges joined after two loads (16.8 M
+// edges: 708 us in one pass, 340 in these three; a first sample of every
+// 16th edge alone takes 680).  Small graphs go in one pass.
+#define UF_SAMPLE1 256
+#define UF_SAMPLE2 16
+#define UF_SAMPLE_MIN (1 << 16)
 __device__ __forceinline__ int32_t ld_par(const int32_t* p) { return *(volatile const int32_t*)p; }
 
 // Parents only ever point to smaller ids, so every walk ends.
@@ -88,13 +100,18 @@ __global__ void k_uf_init(int32_t* par, int64_t n)
 
 // hook the larger root under the smaller: the final root of a component is
 // its smallest vertex id.  Retries are bounded; giving up flags an error.
-__global__ void k_uf_hook(const uint64_t* __restrict__ keys, int64_t m, int nb, int32_t* par, uint32_t* flags)
+// Takes every `stride`-th edge.
+__global__ void k_uf_hook(const uint64_t* __restrict__ keys, int64_t m, int stride, int nb, int32_t* par,
+                          uint32_t* flags)
 {
     uint64_t mask = (1ull << nb) - 1ull;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * stride; i < m;
+         i += (int64_t)gridDim.x * blockDim.x * stride) {
         uint64_t k = keys[i];
-        int32_t a = uf_find(par, (int32_t)(k >> (nb + 1)));
-        int32_t b = uf_find(par, (int32_t)((k >> 1) & mask));
+        int32_t a = (int32_t)(k >> (nb + 1)), b = (int32_t)((k >> 1) & mask);
+        if (ld_par(par + a) == ld_par(par + b)) continue;  // one parent: joined already
+        a = uf_find(par, a);
+        b = uf_find(par, b);
         int tries = 0;
         while (a != b) {
             if (a > b) {
@@ -114,12 +131,21 @@ __global__ void k_uf_hook(const uint64_t* __restrict__ keys, int64_t m, int nb, 
     }
 }
 
+// every vertex points at its root; sizes of the components (nullable), one
+// atomic per warp and root (nearly all vertices share one)
 __global__ void k_uf_sizes(int32_t* par, int64_t n, int32_t* size)
 {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        int32_t r = uf_find(par, (int32_t)v);
+        // a climb that writes nothing: another thread's path halving could
+        // otherwise put an inner ancestor back after this vertex's root
+        int32_t r = (int32_t)v;
+        for (int32_t p = ld_par(par + r); p != r; p = ld_par(par + r)) r = p;
         par[v] = r;
-        atomicAdd(size + r, 1);
+        if (size) {
+            const unsigned act = __activemask();
+            const unsigned same = __match_any_sync(act, r);
+            if ((threadIdx.x & 31) == __ffs((int)same) - 1) atomicAdd(size + r, __popc(same));
+        }
     }
 }
 
@@ -161,8 +187,7 @@ __global__ void k_keep_edges(const uint64_t* __restrict__ keys, int64_t m, int n
 // final edge list + lower-triangle keys (v, u, neg) for the CSR transpose
 __global__ void k_emit_edges(const uint64_t* __restrict__ keys, int64_t m, int nb, const int32_t* __restrict__ ekeep,
                              const int32_t* __restrict__ epos, const int32_t* __restrict__ newid, int nb2,
-                             int2* __restrict__ edges, uint64_t* __restrict__ lkeys, int32_t* __restrict__ deg,
-                             int32_t* __restrict__ updeg)
+                             int2* __restrict__ edges, uint64_t* __restrict__ lkeys)
 {
     uint64_t mask = (1ull << nb) - 1ull;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
@@ -173,44 +198,84 @@ __global__ void k_emit_edges(const uint64_t* __restrict__ keys, int64_t m, int n
         int32_t p = epos[i];
         edges[p] = make_int2(u, (int32_t)((uint32_t)v | (neg << 31)));
         lkeys[p] = ((uint64_t)v << (nb2 + 1)) | ((uint64_t)u << 1) | neg;
-        atomicAdd(deg + u, 1);
-        atomicAdd(deg + v, 1);
-        atomicAdd(updeg + u, 1);
     }
 }
 
-// upper part of row u: neighbours v > u, in edge order (ascending v)
-__global__ void k_fill_upper(const int2* __restrict__ edges, int64_t m, const int32_t* __restrict__ rowptr,
-                             const int32_t* __restrict__ deg, const int32_t* __restrict__ updeg,
-                             const int32_t* __restrict__ ufirst, int32_t* __restrict__ col)
+// The edges are sorted by u and the lower keys by v, so the first position of
+// every vertex in either follows from where neighbours differ (no counting
+// atomics, which the hubs would serialise):
+//   ufirst[x], lfirst[x] = first edge with u >= x, first key with v >= x
+// (n + 1 entries).  A row is its lower neighbours, then its upper ones, so
+//   rowptr[x] = ufirst[x] + lfirst[x],
+//   entry of edge i in row u   = lfirst[u + 1] + i,
+//   entry of key p in row v    = ufirst[v] + p.
+__global__ void k_first(const int2* __restrict__ edges, const uint64_t* __restrict__ lkeys, int64_t m, int64_t n, int nb2,
+                        int32_t* __restrict__ ufirst, int32_t* __restrict__ lfirst)
 {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= m; i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t a = i > 0 ? edges[i - 1].x : -1, b = i < m ? edges[i].x : n;
+        for (int64_t x = a + 1; x <= b; x++) ufirst[x] = (int32_t)i;
+        a = i > 0 ? (int64_t)(lkeys[i - 1] >> (nb2 + 1)) : -1;
+        b = i < m ? (int64_t)(lkeys[i] >> (nb2 + 1)) : n;
+        for (int64_t x = a + 1; x <= b; x++) lfirst[x] = (int32_t)i;
+    }
+}
+
+__global__ void k_rowptr(const int32_t* __restrict__ ufirst, const int32_t* __restrict__ lfirst, int64_t n,
+                         int32_t* __restrict__ rowptr, int32_t* __restrict__ deg)
+{
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t r = ufirst[v] + lfirst[v];
+        rowptr[v] = r;
+        if (v < n) deg[v] = ufirst[v + 1] + lfirst[v + 1] - r;
+    }
+}
+
+// The scorer takes every edge from its colder endpoint (lower degree; on a
+// tie the larger id) to the hotter one, sorted by (colder, hotter): these are
+// the CSR entries whose row is the colder end, in row order.
+__device__ __forceinline__ bool is_colder(const int32_t* deg, int32_t v, int32_t u)
+{
+    return deg[v] < deg[u] || (deg[v] == deg[u] && v > u);
+}
+
+// upper part of row u: neighbours v > u, in edge order (ascending v); lower
+// part of row v: neighbours u < v, from the (v, u)-sorted keys; and for every
+// entry whether its row is the edge's colder end
+__global__ void k_fill_rows(const int2* __restrict__ edges, const uint64_t* __restrict__ lkeys, int64_t m, int nb2,
+                            const int32_t* __restrict__ ufirst, const int32_t* __restrict__ lfirst,
+                            const int32_t* __restrict__ deg, int32_t* __restrict__ col, int32_t* __restrict__ cold)
+{
+    const uint64_t mask = (1ull << nb2) - 1ull;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        int2 e = edges[i];
-        int32_t u = e.x;
-        int32_t low = deg[u] - updeg[u];
-        col[rowptr[u] + low + (int32_t)(i - ufirst[u])] = e.y;
+        const int2 e = edges[i];
+        const int64_t pu = (int64_t)lfirst[e.x + 1] + i;
+        col[pu] = e.y;
+        cold[pu] = is_colder(deg, e.x, (int32_t)((uint32_t)e.y & SB_ID_MASK)) ? 1 : 0;
+        const uint64_t k = lkeys[i];
+        const int32_t v = (int32_t)(k >> (nb2 + 1)), u = (int32_t)((k >> 1) & mask);
+        const int64_t pv = (int64_t)ufirst[v] + i;
+        col[pv] = (int32_t)((uint32_t)u | ((uint32_t)(k & 1) << 31));
+        cold[pv] = is_colder(deg, v, u) ? 1 : 0;
     }
 }
 
-// lower part of row v: neighbours u < v, from the (v, u)-sorted keys
-__global__ void k_fill_lower(const uint64_t* __restrict__ lkeys, int64_t m, int nb2, const int32_t* __restrict__ rowptr,
-                             const int32_t* __restrict__ lfirst, int32_t* __restrict__ col)
+// the colder-end entries at their positions (exclusive counts of `cold`)
+__global__ void k_emit_sc_edges(const int2* __restrict__ edges, const uint64_t* __restrict__ lkeys, int64_t m, int nb2,
+                                const int32_t* __restrict__ ufirst, const int32_t* __restrict__ lfirst,
+                                const int32_t* __restrict__ cold, const int32_t* __restrict__ pos,
+                                int2* __restrict__ out)
 {
-    uint64_t mask = (1ull << nb2) - 1ull;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t k = lkeys[p];
-        int32_t v = (int32_t)(k >> (nb2 + 1));
-        uint32_t u = (uint32_t)((k >> 1) & mask);
-        uint32_t neg = (uint32_t)(k & 1);
-        col[rowptr[v] + (int32_t)(p - lfirst[v])] = (int32_t)(u | (neg << 31));
+    const uint64_t mask = (1ull << nb2) - 1ull;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        const int2 e = edges[i];
+        const int64_t pu = (int64_t)lfirst[e.x + 1] + i;
+        if (cold[pu]) out[pos[pu]] = e;
+        const uint64_t k = lkeys[i];
+        const int32_t v = (int32_t)(k >> (nb2 + 1));
+        const int64_t pv = (int64_t)ufirst[v] + i;
+        if (cold[pv]) out[pos[pv]] = make_int2(v, (int32_t)((uint32_t)((k >> 1) & mask) | ((uint32_t)(k & 1) << 31)));
     }
-}
-
-__global__ void k_lowdeg(const int32_t* __restrict__ deg, const int32_t* __restrict__ updeg, int64_t n,
-                         int32_t* __restrict__ low)
-{
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        low[v] = deg[v] - updeg[v];
 }
 
 __global__ void k_chunks(const int32_t* __restrict__ deg, int64_t n, int chunk, int32_t* __restrict__ nch,
@@ -232,7 +297,7 @@ __global__ void k_degkeys(const int32_t* __restrict__ deg, int64_t n, uint64_t* 
                           int split_first, int nb)
 {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t hi = split_first ? (deg[v] > chunk ? 0u : 1u) : (0x7FFFFFFFu - (uint32_t)deg[v]);
+        const uint32_t hi = split_first ? (deg[v] > chunk ? 0u : 1u) : ((2u << (nb - 1)) - (uint32_t)deg[v]);
         keys[v] = ((uint64_t)hi << nb) | (uint64_t)v;  // the vertex in the low nb bits
     }
 }
@@ -445,13 +510,16 @@ static sb_status build_items(sb_ctx* c, const int32_t* deg, int64_t n, int chunk
     int32_t* perm = nullptr;
     if (order != 0) {
         uint64_t* keys = T.get<uint64_t>(n);
+        uint64_t* alt = T.get<uint64_t>(n);
         perm = T.get<int32_t>(n);
         int32_t* nch_sorted = T.get<int32_t>(n);
-        if (!keys || !perm || !nch_sorted) return sb_fail(c, SB_ERR_OOM, "item scratch");
+        if (!keys || !alt || !perm || !nch_sorted) return sb_fail(c, SB_ERR_OOM, "item scratch");
         const int nbv = bits_for(n > 1 ? n - 1 : 1);
         k_degkeys<<<g, 256, 0, c->stream>>>(deg, n, keys, chunk, order == 2 ? 1 : 0, nbv);
         SB_TRY(sb_after_launch(c, "k_degkeys"));
-        SB_TRY(sb_radix_sort_u64(c, keys, n, nbv + (order == 2 ? 1 : 31)));
+        // the vertices are in order already: the degree (below n) or the split
+        // bit alone decides, and the sort is stable
+        SB_TRY(sb_radix_sort_u64(c, &keys, &alt, n, nbv, nbv + (order == 2 ? 1 : nbv + 1)));
         k_perm<<<g, 256, 0, c->stream>>>(keys, n, nch, perm, nch_sorted, nbv);
         SB_TRY(sb_after_launch(c, "k_perm"));
         SB_TRY(sb_scan_i32(c, nch_sorted, ipos, n, tot + 0));
@@ -488,29 +556,6 @@ struct BatchIn {
     const int64_t* voff;
     const int64_t* eofs;
 };
-
-// key of the scorer's copy of an edge: (colder << (nb + 1)) | (hotter << 1) | neg,
-// colder = the endpoint of lower degree (on a tie, the larger id)
-__global__ void k_orient_keys(const int2* __restrict__ edges, int64_t m, const int32_t* __restrict__ deg, int nb,
-                              uint64_t* __restrict__ keys)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const int2 ed = edges[e];
-        const uint32_t u = (uint32_t)ed.x, v = (uint32_t)ed.y & SB_ID_MASK;
-        const bool u_cold = deg[u] < deg[v];  // u < v, so a tie makes v the colder one
-        const uint64_t cold = u_cold ? u : v, hot = u_cold ? v : u;
-        keys[e] = (cold << (nb + 1)) | (hot << 1) | (uint64_t)(ed.y < 0 ? 1 : 0);
-    }
-}
-
-__global__ void k_emit_sc_edges(const uint64_t* __restrict__ keys, int64_t m, int nb, int2* __restrict__ out)
-{
-    const uint64_t idm = (1ull << nb) - 1ull;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = keys[e];
-        out[e] = make_int2((int32_t)(k >> (nb + 1)), (int32_t)((uint32_t)((k >> 1) & idm) | ((uint32_t)(k & 1ull) << 31)));
-    }
-}
 
 static sb_status load_graph_impl(sb_ctx* c, int64_t n, int64_t m, const int32_t* src, const int32_t* dst,
                                  const int8_t* sign, uint32_t flags, int64_t* n_out, int64_t* m_out,
@@ -559,7 +604,9 @@ static sb_status load_graph_impl(sb_ctx* c, int64_t n, int64_t m, const int32_t*
         if (code == ERRC_SELF) return sb_fail(c, SB_ERR_SELF_LOOP, "edge %lld is a self-loop", idx);
         return sb_fail(c, SB_ERR_BAD_SIGN, "edge %lld: sign is not +1/-1", idx);
     }
-    SB_TRY(sb_radix_sort_u64(c, keys, m, 2 * nb + 1));
+    uint64_t* alt = T.get<uint64_t>(m);
+    if (!alt) return sb_fail(c, SB_ERR_OOM, "ingest scratch");
+    SB_TRY(sb_radix_sort_u64(c, &keys, &alt, m, 1, 2 * nb + 1));  // by pair; k_heads sees either order of the signs
     int32_t* head = T.get<int32_t>(m);
     int32_t* hpos = T.get<int32_t>(m);
     if (!head || !hpos) return sb_fail(c, SB_ERR_OOM, "ingest scratch");
@@ -584,8 +631,15 @@ static sb_status load_graph_impl(sb_ctx* c, int64_t n, int64_t m, const int32_t*
     unsigned gm1 = grid_for(c, m1);
     k_uf_init<<<gn, 256, 0, c->stream>>>(par, n);
     SB_CHECK_CUDA(c, cudaMemsetAsync(size, 0, sizeof(int32_t) * n, c->stream));
-    k_uf_hook<<<gm1, 256, 0, c->stream>>>(ukeys, m1, nb, par, flags_d);
-    SB_TRY(sb_after_launch(c, "k_uf_hook"));
+    for (int stride : {UF_SAMPLE1, UF_SAMPLE2, 1}) {
+        if (stride > 1 && m1 < UF_SAMPLE_MIN) continue;
+        k_uf_hook<<<grid_for(c, sb_cdiv(m1, stride)), 256, 0, c->stream>>>(ukeys, m1, stride, nb, par, flags_d);
+        SB_TRY(sb_after_launch(c, "k_uf_hook"));
+        if (stride > 1) {
+            k_uf_sizes<<<gn, 256, 0, c->stream>>>(par, n, nullptr);
+            SB_TRY(sb_after_launch(c, "k_uf_sizes"));
+        }
+    }
     k_uf_sizes<<<gn, 256, 0, c->stream>>>(par, n, size);
     SB_TRY(sb_after_launch(c, "k_uf_sizes"));
     int32_t* keep = T.get<int32_t>(n);
@@ -648,43 +702,33 @@ static sb_status load_graph_impl(sb_ctx* c, int64_t n, int64_t m, const int32_t*
     c->rowptr = (int32_t*)sb_dalloc(c, sizeof(int32_t) * (size_t)(n1 + 1));
     c->col = (int32_t*)sb_dalloc(c, sizeof(int32_t) * (size_t)(2 * m2 > 0 ? 2 * m2 : 1));
     c->vweight = (uint64_t*)sb_dalloc(c, sizeof(uint64_t) * (size_t)n1);
-    uint64_t* lkeys = T.get<uint64_t>(m2);
+    uint64_t* lkeys = keys;  // the sort's two buffers again: the unique keys are a copy
     int32_t* deg = T.get<int32_t>(n1);
-    int32_t* updeg = T.get<int32_t>(n1);
-    int32_t* ufirst = T.get<int32_t>(n1);
-    int32_t* low = T.get<int32_t>(n1);
-    int32_t* lfirst = T.get<int32_t>(n1);
-    if (!c->edges || !c->rowptr || !c->col || !c->vweight || !lkeys || !deg || !updeg || !ufirst || !low || !lfirst)
-        return sb_fail(c, SB_ERR_OOM, "graph storage");
-    SB_CHECK_CUDA(c, cudaMemsetAsync(deg, 0, sizeof(int32_t) * n1, c->stream));
-    SB_CHECK_CUDA(c, cudaMemsetAsync(updeg, 0, sizeof(int32_t) * n1, c->stream));
-    k_emit_edges<<<gm1, 256, 0, c->stream>>>(ukeys, m1, nb, ekeep, epos, newid, nb2, c->edges, lkeys, deg, updeg);
-    SB_TRY(sb_after_launch(c, "k_emit_edges"));
-    SB_TRY(sb_scan_i32(c, deg, c->rowptr, n1, tot + 3));
-    // rowptr[n1] = 2 m2
-    int32_t last = (int32_t)(2 * m2);
-    SB_CHECK_CUDA(c, cudaMemcpyAsync(c->rowptr + n1, &last, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
-    SB_TRY(sb_scan_i32(c, updeg, ufirst, n1, nullptr));
-    unsigned gm2 = grid_for(c, m2), gn1 = grid_for(c, n1);
-    k_fill_upper<<<gm2, 256, 0, c->stream>>>(c->edges, m2, c->rowptr, deg, updeg, ufirst, c->col);
-    SB_TRY(sb_after_launch(c, "k_fill_upper"));
-    SB_TRY(sb_radix_sort_u64(c, lkeys, m2, 2 * nb2 + 1));
-    k_lowdeg<<<gn1, 256, 0, c->stream>>>(deg, updeg, n1, low);
-    SB_TRY(sb_after_launch(c, "k_lowdeg"));
-    SB_TRY(sb_scan_i32(c, low, lfirst, n1, nullptr));
-    k_fill_lower<<<gm2, 256, 0, c->stream>>>(lkeys, m2, nb2, c->rowptr, lfirst, c->col);
-    SB_TRY(sb_after_launch(c, "k_fill_lower"));
-    // scorer stream: every edge from its colder endpoint (lower degree) to
-    // the hotter one, sorted by (colder, hotter); two zero edges of padding
-    // let tile copies round their size up to 16 bytes
+    int32_t* ufirst = T.get<int32_t>(n1 + 1);
+    int32_t* lfirst = T.get<int32_t>(n1 + 1);
+    int32_t* cold = T.get<int32_t>(2 * m2);
+    int32_t* cpos = T.get<int32_t>(2 * m2);
+    // two zero edges of padding let the scorer's tile copies round their size
+    // up to 16 bytes
     c->sc_edges = (int2*)sb_dalloc(c, sizeof(int2) * (size_t)(m2 + 2));
-    if (!c->sc_edges) return sb_fail(c, SB_ERR_OOM, "graph storage");
+    if (!c->edges || !c->rowptr || !c->col || !c->vweight || !c->sc_edges || !deg || !ufirst || !lfirst ||
+        !cold || !cpos)
+        return sb_fail(c, SB_ERR_OOM, "graph storage");
+    k_emit_edges<<<gm1, 256, 0, c->stream>>>(ukeys, m1, nb, ekeep, epos, newid, nb2, c->edges, lkeys);
+    SB_TRY(sb_after_launch(c, "k_emit_edges"));
+    unsigned gm2 = grid_for(c, m2 + 1), gn1 = grid_for(c, n1 + 1);
+    // by v alone: the keys come in (u, v) order and the sort is stable
+    SB_TRY(sb_radix_sort_u64(c, &lkeys, &alt, m2, nb2 + 1, 2 * nb2 + 1));
+    k_first<<<gm2, 256, 0, c->stream>>>(c->edges, lkeys, m2, n1, nb2, ufirst, lfirst);
+    SB_TRY(sb_after_launch(c, "k_first"));
+    k_rowptr<<<gn1, 256, 0, c->stream>>>(ufirst, lfirst, n1, c->rowptr, deg);
+    SB_TRY(sb_after_launch(c, "k_rowptr"));
     SB_CHECK_CUDA(c, cudaMemsetAsync(c->sc_edges + m2, 0, 2 * sizeof(int2), c->stream));
     if (m2 > 0) {
-        k_orient_keys<<<gm2, 256, 0, c->stream>>>(c->edges, m2, deg, nb2, lkeys);
-        SB_TRY(sb_after_launch(c, "k_orient_keys"));
-        SB_TRY(sb_radix_sort_u64(c, lkeys, m2, 2 * nb2 + 1));
-        k_emit_sc_edges<<<gm2, 256, 0, c->stream>>>(lkeys, m2, nb2, c->sc_edges);
+        k_fill_rows<<<gm2, 256, 0, c->stream>>>(c->edges, lkeys, m2, nb2, ufirst, lfirst, deg, c->col, cold);
+        SB_TRY(sb_after_launch(c, "k_fill_rows"));
+        SB_TRY(sb_scan_i32(c, cold, cpos, 2 * m2, nullptr));
+        k_emit_sc_edges<<<gm2, 256, 0, c->stream>>>(c->edges, lkeys, m2, nb2, ufirst, lfirst, cold, cpos, c->sc_edges);
         SB_TRY(sb_after_launch(c, "k_emit_sc_edges"));
     }
     if (B) {

@@ -272,8 +272,9 @@ void sb_release_graphl(sb_ctx* c);
 
 // exclusive scan of n int32 values into out (int32); returns total via *total_dev (device int64*, nullable)
 sb_status sb_scan_i32(sb_ctx* c, const int32_t* in, int32_t* out, int64_t n, int64_t* total_dev);
-// LSD radix sort of uint64 keys over the low `bits` bits; result in keys
-sb_status sb_radix_sort_u64(sb_ctx* c, uint64_t* keys, int64_t n, int bits);
+// stable LSD radix sort of n uint64 keys by their bits [lo, hi), alternating
+// between two buffers: the result is in *keys afterwards
+sb_status sb_radix_sort_u64(sb_ctx* c, uint64_t** keys, uint64_t** alt, int64_t n, int lo, int hi);
 
 // entry points implemented per translation unit
 sb_status sb_cloud_insert_batch(sb_ctx* c);
