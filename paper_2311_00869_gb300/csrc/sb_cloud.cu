@@ -35,6 +35,7 @@ __global__ void k_cloud_assign(const uint64_t* __restrict__ hashes, const int32_
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int32_t ns = meta[0];
+    meta[2] = 0;
     for (int64_t i = 0; i < K; i++) {
         const uint64_t h = hashes[i];
         const uint64_t key = cl_key(h, hash_bits);
@@ -53,7 +54,7 @@ __global__ void k_cloud_assign(const uint64_t* __restrict__ hashes, const int32_
         if (found >= 0) {
             entries[found].count += 1;
             assign[i] = found;
-            if (entries[found].S != counts[i]) mismatch[i] = 1;  // certainly another state
+            if (entries[found].S != counts[i]) mismatch[i] = meta[2] = 1;  // certainly another state
         } else if (ns >= max_states || probes >= slots) {
             meta[1] += 1;
             assign[i] = -1;
@@ -96,7 +97,10 @@ __global__ void __launch_bounds__(CLP_THREADS)
     __shared__ int32_t s_part[CLP_THREADS / 32], s_ns, s_total;
     const int tid = threadIdx.x;
     const uint64_t mask = (uint64_t)(slots - 1);
-    if (tid == 0) s_ns = meta[0];
+    if (tid == 0) {
+        s_ns = meta[0];
+        meta[2] = 0;
+    }
     for (int i = tid; i < P; i += CLP_THREADS) {
         key[i] = i < K ? cl_key(hashes[i], hash_bits) : ~0ull;
         idx[i] = i < K ? i : 0x7FFFFFFF;
@@ -213,7 +217,7 @@ __global__ void __launch_bounds__(CLP_THREADS)
             continue;
         }
         atomicAdd(&entries[st].count, 1);
-        if (entries[st].S != counts[t]) mismatch[t] = 1;  // certainly another state
+        if (entries[st].S != counts[t]) mismatch[t] = meta[2] = 1;  // certainly another state
     }
     if (tid == 0) meta[0] = (int32_t)min((int64_t)s_ns + s_total, max_states);
 }
@@ -258,6 +262,7 @@ __global__ void k_cloud_assign_scalable(const uint64_t* __restrict__ hashes, con
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int32_t ns = meta[0];
+    meta[2] = 0;
     int32_t maxS = 0, arg = -1;
     auto rescan = [&]() {
         arg = -1;
@@ -287,7 +292,7 @@ __global__ void k_cloud_assign_scalable(const uint64_t* __restrict__ hashes, con
             entries[found].count += 1;
             assign[i] = found;
             touch[found] = 1;
-            if (entries[found].S != counts[i]) mismatch[i] = 1;  // certainly another state
+            if (entries[found].S != counts[i]) mismatch[i] = meta[2] = 1;  // certainly another state
             continue;
         }
         int32_t st;
@@ -339,7 +344,8 @@ __device__ __forceinline__ uint32_t cl_bit(const uint64_t* row, const uint64_t* 
 __global__ void __launch_bounds__(CLV_THREADS)
     k_cloud_verify(const uint64_t* __restrict__ lab, int64_t n, int W, const uint64_t* __restrict__ flipw, int64_t K,
                    const int32_t* __restrict__ slot, const int32_t* __restrict__ assign,
-                   const int32_t* __restrict__ rep, uint64_t* bits, int64_t max_states, int32_t* mismatch)
+                   const int32_t* __restrict__ rep, uint64_t* bits, int64_t max_states, int32_t* mismatch,
+                   int32_t* meta)
 {
     extern __shared__ uint64_t rows[];  // 64 x W
     const int64_t chunk = blockIdx.x;
@@ -375,7 +381,7 @@ __global__ void __launch_bounds__(CLV_THREADS)
         } else {
             const int sc = creator < 0 ? 0 : slot ? slot[creator] : creator;
             const uint64_t other = creator >= 0 ? rows[(sc & 63) * W + (sc >> 6)] : *stored;
-            if (other != col) mismatch[i] = 1;
+            if (other != col) mismatch[i] = meta[2] = 1;
         }
     }
 }
@@ -399,26 +405,21 @@ __global__ void k_cloud_pair(const uint64_t* __restrict__ lab, int64_t n, int W,
     }
 }
 
-__global__ void k_cloud_count(const int32_t* __restrict__ mismatch, int64_t K, int32_t* meta)
-{
-    int32_t c = 0;
-    for (int64_t i = threadIdx.x; i < K; i += blockDim.x) c += mismatch[i];
-    for (int d = 16; d; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
-    __shared__ int32_t part[32];
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int32_t t = 0;
-        for (unsigned i = 0; i < blockDim.x / 32; i++) t += part[i];
-        meta[2] = t;
-    }
-}
-
 __global__ void k_cloud_gather(const uint64_t* __restrict__ bits, int64_t nchunks, int64_t max_states, int64_t s,
                                uint64_t* out)
 {
     for (int64_t ch = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ch < nchunks; ch += (int64_t)gridDim.x * blockDim.x)
         out[ch] = bits[ch * max_states + s];
+}
+
+static sb_status cloud_clear(sb_ctx* c)
+{
+    // empty slots: state = -1 (all bytes 0xFF)
+    SB_CHECK_CUDA(c, cudaMemsetAsync(c->cl_table, 0xFF, sizeof(sb_cloud_slot) * (size_t)c->cl_slots, c->stream));
+    SB_CHECK_CUDA(c, cudaMemsetAsync(c->cl_meta, 0, sizeof(int32_t) * 8, c->stream));
+    c->cl_n_host = 0;
+    c->cl_order.clear();
+    return SB_OK;
 }
 
 sb_status sb_cloud_alloc(sb_ctx* c)
@@ -443,17 +444,13 @@ sb_status sb_cloud_alloc(sb_ctx* c)
         sb_release_cloud(c);
         return sb_fail(c, SB_ERR_OOM, "cloud storage (%lld states)", (long long)c->cl_max);
     }
-    // empty slots: state = -1 (all bytes 0xFF)
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->cl_table, 0xFF, sizeof(sb_cloud_slot) * (size_t)slots, c->stream));
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->cl_meta, 0, sizeof(int32_t) * 8, c->stream));
-    c->cl_n_host = 0;
-    return SB_OK;
+    return cloud_clear(c);
 }
 
 // Rare path: trees whose hash matched a different state.  Each is re-probed
 // on the host with an exact device comparison against every state sharing
 // its key, and gets a new state when none is equal.
-static sb_status cloud_resolve_collisions(sb_ctx* c)
+static sb_status cloud_resolve_collisions(sb_ctx* c, int32_t* meta_out)
 {
     const int64_t K = c->K;
     std::vector<int32_t> assign(K), mism(K);
@@ -529,10 +526,12 @@ static sb_status cloud_resolve_collisions(sb_ctx* c)
     meta[2] = 0;
     SB_CHECK_CUDA(c, cudaMemcpyAsync(c->cl_meta, meta, sizeof(int32_t) * 4, cudaMemcpyHostToDevice, c->stream));
     SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
+    memcpy(meta_out, meta, sizeof(int32_t) * 4);
     return SB_OK;
 }
 
-sb_status sb_cloud_insert_batch(sb_ctx* c)
+// meta_out (host, 4 words, nullable): the cloud's counters afterwards
+sb_status sb_cloud_insert_batch(sb_ctx* c, int32_t* meta_out)
 {
     if (c->batch_in_cloud) return SB_OK;
     SB_TRY(sb_cloud_alloc(c));
@@ -569,10 +568,8 @@ sb_status sb_cloud_insert_batch(sb_ctx* c)
     const int32_t* slot = c->ordered ? c->order + 64 * (int64_t)c->W : nullptr;
     k_cloud_verify<<<(unsigned)nchunks, CLV_THREADS, smem, c->stream>>>(c->labels, c->n, c->W, c->flipw, c->K, slot,
                                                                          c->cl_assign, c->cl_rep, c->cl_bits,
-                                                                         c->cl_max, c->cl_mismatch);
+                                                                         c->cl_max, c->cl_mismatch, c->cl_meta);
     SB_TRY(sb_after_launch(c, "k_cloud_verify"));
-    k_cloud_count<<<1, 1024, 0, c->stream>>>(c->cl_mismatch, c->K, c->cl_meta);
-    SB_TRY(sb_after_launch(c, "k_cloud_count"));
     int32_t meta[4];
     SB_CHECK_CUDA(c, cudaMemcpyAsync(meta, c->cl_meta, sizeof(meta), cudaMemcpyDeviceToHost, c->stream));
     SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -580,9 +577,10 @@ sb_status sb_cloud_insert_batch(sb_ctx* c)
         // a 64-bit hash shared by two different states: resolved exactly by the
         // unbounded cloud; the scalable one reports it instead
         if (c->cl_fmax > 0) return sb_fail(c, SB_ERR_DEVICE_CHECK, "state hash collision in the scalable cloud");
-        SB_TRY(cloud_resolve_collisions(c));
+        SB_TRY(cloud_resolve_collisions(c, meta));
     }
     c->batch_in_cloud = true;
+    if (meta_out) memcpy(meta_out, meta, sizeof(meta));
     return SB_OK;
 }
 
@@ -590,12 +588,18 @@ extern "C" sb_status sb_cloud_reset(sb_ctx* c, int64_t max_states, int32_t hash_
 {
     if (!c || max_states < 0 || max_states > (1ll << 30) || hash_bits < 0 || hash_bits > 64) return SB_ERR_ARG;
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
-    SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
-    sb_release_cloud(c);
-    c->cl_max = max_states > 0 ? max_states : CL_DEFAULT_STATES;
+    const int64_t want = max_states > 0 ? max_states : CL_DEFAULT_STATES;
+    // the same capacity on the same graph keeps its buffers
+    const bool keep = c->cl_table && c->cl_max == want;
+    if (!keep) {
+        SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
+        sb_release_cloud(c);
+        c->cl_max = want;
+    }
     c->cl_hash_bits = hash_bits > 0 ? hash_bits : 64;
     c->cl_fmax = 0;
     c->batch_in_cloud = true;  // a reset starts from the next sampled batch
+    if (keep) return cloud_clear(c);
     if (c->has_graph) SB_TRY(sb_cloud_alloc(c));
     return SB_OK;
 }
@@ -614,10 +618,20 @@ extern "C" sb_status sb_cloud(sb_ctx* c, sb_cloud_entry* out, int64_t cap, int64
     if (!c->has_graph) return sb_fail(c, SB_ERR_STATE, "no graph loaded");
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
     SB_TRY(sb_cloud_alloc(c));
-    if (c->has_batch && !c->batch_in_cloud) SB_TRY(sb_cloud_insert_batch(c));
     int32_t meta[4];
-    SB_CHECK_CUDA(c, cudaMemcpyAsync(meta, c->cl_meta, sizeof(meta), cudaMemcpyDeviceToHost, c->stream));
-    SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
+    std::vector<sb_cloud_entry> host;
+    const bool insert = c->has_batch && !c->batch_in_cloud;
+    if (insert) SB_TRY(sb_cloud_insert_batch(c, meta));
+    if (!insert || out || fr_min_out) {
+        // the counters and, as far as the caller has room, the entries: one wait
+        const int64_t ask = std::min<int64_t>({cap, c->cl_max, CL_DEFAULT_STATES});
+        host.resize(ask);
+        SB_CHECK_CUDA(c, cudaMemcpyAsync(meta, c->cl_meta, sizeof(meta), cudaMemcpyDeviceToHost, c->stream));
+        if (ask > 0)
+            SB_CHECK_CUDA(c, cudaMemcpyAsync(host.data(), c->cl_entries, sizeof(sb_cloud_entry) * (size_t)ask,
+                                             cudaMemcpyDeviceToHost, c->stream));
+        SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
+    }
     const int64_t ns = meta[0];
     c->cl_n_host = ns;
     *n_states_out = ns;
@@ -626,9 +640,11 @@ extern "C" sb_status sb_cloud(sb_ctx* c, sb_cloud_entry* out, int64_t cap, int64
         return full ? sb_fail(c, SB_ERR_CLOUD_FULL, "cloud capacity %lld reached; %d trees not stored",
                               (long long)c->cl_max, meta[1])
                     : SB_OK;
-    std::vector<sb_cloud_entry> host(ns > 0 ? ns : 1);
-    if (ns > 0)
-        SB_CHECK_CUDA(c, cudaMemcpy(host.data(), c->cl_entries, sizeof(sb_cloud_entry) * ns, cudaMemcpyDeviceToHost));
+    const int64_t have = (int64_t)host.size();
+    host.resize(ns > 0 ? ns : 1);
+    if (ns > have)
+        SB_CHECK_CUDA(c, cudaMemcpy(host.data() + have, c->cl_entries + have, sizeof(sb_cloud_entry) * (ns - have),
+                                    cudaMemcpyDeviceToHost));
     // order of first appearance (states created on the collision path are
     // numbered after the states of later trees of their batch)
     c->cl_order.resize(ns);
@@ -645,7 +661,10 @@ extern "C" sb_status sb_cloud(sb_ctx* c, sb_cloud_entry* out, int64_t cap, int64
     if (k > 0) {
         std::vector<sb_cloud_entry> sorted(k);
         for (int64_t i = 0; i < k; i++) sorted[i] = host[c->cl_order[i]];
-        SB_CHECK_CUDA(c, cudaMemcpy(out, sorted.data(), sizeof(sb_cloud_entry) * k, cudaMemcpyDefault));
+        if (sb_is_device_ptr(out))
+            SB_CHECK_CUDA(c, cudaMemcpy(out, sorted.data(), sizeof(sb_cloud_entry) * k, cudaMemcpyHostToDevice));
+        else
+            memcpy(out, sorted.data(), sizeof(sb_cloud_entry) * (size_t)k);
     }
     if (full)
         return sb_fail(c, SB_ERR_CLOUD_FULL, "cloud capacity %lld reached; %d trees not stored", (long long)c->cl_max,
@@ -667,7 +686,7 @@ static sb_status cloud_state_dev(sb_ctx* c, int64_t idx, uint64_t** out)
     *out = nullptr;
     if (!c->has_graph || !c->cl_table) return sb_fail(c, SB_ERR_STATE, "no cloud");
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
-    if (c->has_batch && !c->batch_in_cloud) SB_TRY(sb_cloud_insert_batch(c));
+    if (c->has_batch && !c->batch_in_cloud) SB_TRY(sb_cloud_insert_batch(c, nullptr));
     int32_t ns = 0;
     SB_CHECK_CUDA(c, cudaMemcpyAsync(&ns, c->cl_meta, sizeof(ns), cudaMemcpyDeviceToHost, c->stream));
     SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -277,7 +277,7 @@ sb_status sb_scan_i32(sb_ctx* c, const int32_t* in, int32_t* out, int64_t n, int
 sb_status sb_radix_sort_u64(sb_ctx* c, uint64_t** keys, uint64_t** alt, int64_t n, int lo, int hi);
 
 // entry points implemented per translation unit
-sb_status sb_cloud_insert_batch(sb_ctx* c);
+sb_status sb_cloud_insert_batch(sb_ctx* c, int32_t* meta_out);
 sb_status sb_cloud_alloc(sb_ctx* c);
 sb_status sb_score_batch(sb_ctx* c);
 // sampled-batch storage for trees [tree_begin, tree_begin + K) (labels,
