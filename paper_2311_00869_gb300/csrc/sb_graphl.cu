@@ -90,12 +90,13 @@ struct GlCols {
 #pragma unroll
         for (int k = 0; k < VEC; k++) mx[k] = 0;
     }
-    __device__ __forceinline__ void flush(const GlArgs& A, int r0, uint32_t* smax)
+    // columns r0, r0 + stride, ..
+    __device__ __forceinline__ void flush(const GlArgs& A, int r0, int stride, uint32_t* smax)
     {
         if (g < 0) return;
 #pragma unroll
         for (int k = 0; k < VEC; k++) {
-            const int r = r0 + k;
+            const int r = r0 + k * stride;
             if (r < A.R && mx[k]) atomicMax(A.vgid ? A.colmax + g * A.R + r : smax + r, mx[k]);
         }
     }
@@ -130,10 +131,15 @@ __device__ __forceinline__ float gl_value(const GlArgs& A, float x, float scale_
 // (fma.rn.f32x2 by the edge's sign instead of a sign flip and an add per
 // column), and leaves the discrete loss, which took five integer operations
 // per element here, to k_gl_count: this kernel only writes the sign words of
-// its output.  Traced step on the 2^20 R-MAT graph, 256 columns: 4.58 -> 2.98 ms
+// its output.  More rows in flight than that is slower (6 or 8 in registers,
+// or 16 per warp through a cp.async ring in shared memory: 3.4-4.0 ms against
+// 2.93 for the step below): 11.6 TB/s of gathered rows out of L2, a third of
+// them from DRAM, is what the memory system gives.  Rows that are not 16-byte
+// aligned (R not a multiple of 4) are taken in 32-column pieces, up to four
+// per lane (STRIDED): at 37 columns 2.05 -> 1.26 ms a step.  Traced step on the 2^20 R-MAT graph, 256 columns: 4.58 -> 2.98 ms
 // (and 0.12 for k_gl_count); 64 columns without a trace: 1.47 -> 0.89 ms.
-template <int VEC, int SL, bool STEP, int IB>
-__global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlArgs A)
+template <int VEC, int SL, bool STRIDED, bool STEP, int IB>
+__global__ void __launch_bounds__(GL_THREADS, STRIDED && VEC > 1 ? 4 : GL_ROWS_MIN_BLOCKS) k_gl_rows(GlArgs A)
 {
     extern __shared__ uint32_t smax[];  // R (STEP)
     const int R = A.R;
@@ -153,7 +159,9 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
     const int64_t nsplit = A.n_split_items;
     const int64_t nunits = nsplit + sb_cdiv(A.n_items - nsplit, IB);
     for (int seg = 0; seg < nseg; seg++) {
-        const int r0 = seg * seg_w + sl * VEC;
+        // a lane's columns: VEC adjacent ones, or every 32nd from r0 on
+        constexpr int CS = STRIDED ? 32 : 1;
+        const int r0 = STRIDED ? seg * seg_w + sl : seg * seg_w + sl * VEC;
         const bool act = r0 < R;
         GlCols<VEC> cols;
         for (int64_t wu = sub_id; wu < nunits; wu += subs_total)
@@ -164,7 +172,7 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
             const int64_t v = q.x;
             const int64_t g = A.vgid ? A.vgid[v] : 0;
             if (STEP && g != cols.g) {
-                if (act) cols.flush(A, r0, smax);
+                if (act) cols.flush(A, r0, CS, smax);
                 cols.reset(g);
             }
             float acc[VEC];
@@ -174,7 +182,9 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
             for (int j0 = q.y; j0 < q.z; j0 += 32) {
                 const int cnt = min(32, q.z - j0);
                 uint64_t b01 = 0, b23 = 0;
-                float b0 = 0.f;
+                float bs[STRIDED ? VEC : 1];
+#pragma unroll
+                for (int k = 0; k < (STRIDED ? VEC : 1); k++) bs[k] = 0.f;
                 for (int jj = 0; jj < cnt; jj += SL) {
                     const int cc_n = min(SL, cnt - jj);
                     const uint32_t mycol = sl < cc_n ? (uint32_t)__ldg(A.col + j0 + jj + sl) : 0u;
@@ -182,7 +192,7 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
                         uint32_t cc[GL_INFLIGHT];
 #pragma unroll
                         for (int i = 0; i < GL_INFLIGHT; i++) cc[i] = __shfl_sync(smask, mycol, (q0 + i) & (SL - 1), SL);
-                        if constexpr (VEC == 4) {
+                        if constexpr (!STRIDED) {
                             ulonglong2 x[GL_INFLIGHT];
 #pragma unroll
                             for (int i = 0; i < GL_INFLIGHT; i++)
@@ -197,32 +207,42 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
                                     add_signed2(b23, x[i].y, ss);
                                 }
                         } else {
-                            float x[GL_INFLIGHT];
+                            float x[GL_INFLIGHT][VEC];
+#pragma unroll
+                            for (int i = 0; i < GL_INFLIGHT; i++) {
+                                const float* p = A.gin + (int64_t)(cc[i] & SB_ID_MASK) * R + r0;
+#pragma unroll
+                                for (int k = 0; k < VEC; k++)
+                                    if (r0 + CS * k < R && q0 + i < cc_n) x[i][k] = __ldg(p + CS * k);
+                            }
 #pragma unroll
                             for (int i = 0; i < GL_INFLIGHT; i++)
-                                if (act && q0 + i < cc_n) x[i] = __ldg(A.gin + (int64_t)(cc[i] & SB_ID_MASK) * R + r0);
 #pragma unroll
-                            for (int i = 0; i < GL_INFLIGHT; i++)
-                                if (act && q0 + i < cc_n) b0 += flip_sign(x[i], cc[i] & 0x80000000u);
+                                for (int k = 0; k < VEC; k++)
+                                    if (r0 + CS * k < R && q0 + i < cc_n)
+                                        bs[STRIDED ? k : 0] += flip_sign(x[i][k], cc[i] & 0x80000000u);
                         }
                     }
                 }
-                if constexpr (VEC == 4) {
+                if constexpr (!STRIDED) {
                     acc[0] += lo2(b01);
                     acc[1 % VEC] += hi2(b01);
                     acc[2 % VEC] += lo2(b23);
                     acc[3 % VEC] += hi2(b23);
                 } else {
-                    acc[0] += b0;
+#pragma unroll
+                    for (int k = 0; k < VEC; k++) acc[k] += bs[STRIDED ? k : 0];
                 }
             }
             if (q.w >= 0) {
                 const int64_t slot = A.hub_first[q.w] + (q.y - A.rowptr[v]) / SB_GL_CHUNK;
                 if (act) {
-                    if constexpr (VEC == 4)
+                    if constexpr (!STRIDED)
                         *(float4*)(A.partial + slot * R + r0) = make_float4(acc[0], acc[1 % VEC], acc[2 % VEC], acc[3 % VEC]);
                     else
-                        A.partial[slot * R + r0] = acc[0];
+#pragma unroll
+                        for (int k = 0; k < VEC; k++)
+                            if (r0 + CS * k < R) A.partial[slot * R + r0 + CS * k] = acc[k];
                 }
                 continue;
             }
@@ -230,7 +250,7 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
             if (act) {
                 const float* pin = A.gin + v * R + r0;
                 const float* pup = (STEP ? A.scale : A.upstream) + g * R + r0;
-                if (VEC == 4 && A.vec_out) {
+                if (!STRIDED && A.vec_out) {
                     const float4 up = *(const float4*)pup;
                     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (STEP) x = __ldg((const float4*)pin);
@@ -242,8 +262,10 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
                 } else {
 #pragma unroll
                     for (int k = 0; k < VEC; k++) {
-                        out[k] = gl_value<STEP>(A, STEP ? __ldg(pin + k) : 0.f, pup[k], acc[k]);
-                        A.gout_rows[v * R + r0 + k] = out[k];
+                        out[k] = 0.f;
+                        if (r0 + CS * k >= R) continue;
+                        out[k] = gl_value<STEP>(A, STEP ? __ldg(pin + CS * k) : 0.f, pup[CS * k], acc[k]);
+                        A.gout_rows[v * R + r0 + CS * k] = out[k];
                     }
                 }
                 if (STEP) {
@@ -252,19 +274,22 @@ __global__ void __launch_bounds__(GL_THREADS, GL_ROWS_MIN_BLOCKS) k_gl_rows(GlAr
                 }
             }
             if (STEP && A.signs) {
-                if constexpr (VEC == 4) {
+                if constexpr (!STRIDED) {
                     uint32_t w = 0;  // sign word of this lane's 8-lane group
 #pragma unroll
                     for (int k = 0; k < 4; k++)
                         w |= ((__ballot_sync(smask, act && is_neg(out[k % VEC])) >> (lane & ~7)) & 255u) << (8 * k);
                     if (act && (sl & 7) == 0) A.signs[v * A.sign_words + r0 / 32] = w;
                 } else {
-                    const uint32_t w = sign_word(act && is_neg(out[0]), R % 4 == 0);
-                    if (lane == 0) A.signs[v * A.sign_words + r0 / 32] = w;
+#pragma unroll
+                    for (int k = 0; k < VEC; k++) {
+                        const uint32_t w = sign_word(r0 + 32 * k < R && is_neg(out[k]), R % 4 == 0);
+                        if (lane == 0 && r0 + 32 * k < R) A.signs[v * A.sign_words + r0 / 32 + k] = w;
+                    }
                 }
             }
         }
-        if (STEP && act) cols.flush(A, r0, smax);
+        if (STEP && act) cols.flush(A, r0, CS, smax);
     }
     if (STEP) {
         __syncthreads();
@@ -717,12 +742,15 @@ static GlArgs gl_args(sb_ctx* c, int R)
 }
 
 template <bool STEP, int IB>
-static const void* gl_rows_kernel(bool vec4, int64_t lanes)
+static const void* gl_rows_kernel(bool vec4, int64_t lanes, int R)
 {
-    return !vec4        ? (const void*)k_gl_rows<1, 32, STEP, IB>
-           : lanes == 32 ? (const void*)k_gl_rows<4, 32, STEP, IB>
-           : lanes == 16 ? (const void*)k_gl_rows<4, 16, STEP, IB>
-                         : (const void*)k_gl_rows<4, 8, STEP, IB>;
+    if (vec4)
+        return lanes == 32   ? (const void*)k_gl_rows<4, 32, false, STEP, IB>
+               : lanes == 16 ? (const void*)k_gl_rows<4, 16, false, STEP, IB>
+                             : (const void*)k_gl_rows<4, 8, false, STEP, IB>;
+    return R > 64   ? (const void*)k_gl_rows<4, 32, true, STEP, IB>
+           : R > 32 ? (const void*)k_gl_rows<2, 32, true, STEP, IB>
+                    : (const void*)k_gl_rows<1, 32, true, STEP, IB>;
 }
 
 // Lanes per row segment: the knob, or the width whose segments take least in
@@ -744,7 +772,7 @@ static sb_status gl_rows_launch(sb_ctx* c, GlArgs& A)
     const int subs = GL_THREADS / (vec4 && lanes != 32 ? (lanes == 16 ? 16 : 8) : 32);
     const int64_t rows = A.n_items - A.n_split_items;
     const bool small = rows < (int64_t)c->num_sms * GL_ROWS_MIN_BLOCKS * subs * GL_ROWS_PER_SUB;
-    const void* fn = small ? gl_rows_kernel<STEP, 1>(vec4, lanes) : gl_rows_kernel<STEP, GL_ITEM_BLOCK>(vec4, lanes);
+    const void* fn = small ? gl_rows_kernel<STEP, 1>(vec4, lanes, A.R) : gl_rows_kernel<STEP, GL_ITEM_BLOCK>(vec4, lanes, A.R);
     size_t smem = STEP ? sizeof(uint32_t) * (size_t)A.R : 0;
     if (smem > 48 * 1024) SB_CHECK_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
