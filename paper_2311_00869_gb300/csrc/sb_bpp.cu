@@ -60,6 +60,12 @@
 #define BFS_ORDER_MIN (1 << 18)
 // Threads per SM below which a launch spreads its half-words over more lanes.
 #define BFS_SPREAD_THREADS 512
+// Work items below which a graph of mean degree 16 and more does so too, up to
+// 32 lanes per vertex.  Fewest lanes against 32, 128 / 500 trees: 15,000
+// vertices of degree 27 0.77 / 0.98 against 0.57 / 0.68 ms, 95,000 of degree 22
+// 1.24 / 1.35 against 0.91 / 1.20; 180,000 of degree 23 1.19 / 1.87 against
+// 1.57 / 2.06; 100,000 of degree 10 0.60 / 0.83 against 0.83 / 1.04.
+#define BFS_SPREAD_ITEMS (1 << 17)
 #define SYNC_WORDS 48
 // Shared-memory slots: rows of one owner thread's 32 trees (running minima,
 // winner ids), 16-byte aligned, and of one half-word's tree salts.
@@ -881,7 +887,10 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
         G <<= 1;
         ls++;
     }
-    while (Gt == 0 && G < 32 && c->n_items * slices * G < (int64_t)c->num_sms * BFS_SPREAD_THREADS) {
+    // and so does a dense one that fills them a few times over only: its rows
+    // take long, and whole warps hash without a queue
+    const bool dense = c->n_items < BFS_SPREAD_ITEMS && 2 * c->m >= 16 * c->n;
+    while (Gt == 0 && G < 32 && (dense || c->n_items * slices * G < (int64_t)c->num_sms * BFS_SPREAD_THREADS)) {
         G <<= 1;
         ls++;
     }
@@ -1177,8 +1186,13 @@ static sb_status bfs_order(sb_ctx* c)
 static sb_status bfs_enqueue(sb_ctx* c, int32_t* parents_out)
 {
     const int W = c->W, WL = bfs_words_per_launch(c);
-    for (int w0 = 0; w0 < W; w0 += WL) {
-        const int Wb = W - w0 < WL ? W - w0 : WL;
+    for (int w0 = 0, Wb; w0 < W; w0 += Wb) {
+        Wb = W - w0 < WL ? W - w0 : WL;
+        // 17 to 23 words leave most lanes of the second slice idle: 16 words
+        // and the rest apart take less (1100 trees on the 2^20 R-MAT graph 18.6
+        // against 26.4 ms; 1536, 24 words, 27.0 against 28.2, but 2.9 against
+        // 2.7 on 95,000 vertices)
+        if (Wb > 16 && Wb < 24) Wb = 16;
         SB_TRY(run_bfs(c, w0, Wb, parents_out));
     }
     return SB_OK;
