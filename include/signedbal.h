@@ -108,9 +108,10 @@ sb_status sb_profile_read(sb_ctx* ctx, double* ms_out, int64_t* launches_out);
                              16 (64 columns) or 32 (128 columns) when
                              R % 4 == 0 (0 = the width that R suits)
    SB_TUNE_BFS_GROUP         lanes that share one vertex in the BFS, a power
-                             of two in [1, 32]; used when it is more than the
-                             launch's half-words (32 trees each) need (0: by
-                             the size of the graph)
+                             of two in [1, 32]; used when it is one or two
+                             lanes per half-word (32 trees) of the launch,
+                             rounded up to a power of two (otherwise, and at
+                             0, the size of the graph decides)
    SB_TUNE_WAIT_US           limit of every bounded device wait (the BFS grid
                              barrier between levels, the scorer's tile
                              copies), in microseconds at the device's SM

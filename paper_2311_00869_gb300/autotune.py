@@ -3,7 +3,7 @@
 It times the candidate values on the loaded graph with the library's own
 CUDA-event profiler and keeps the fastest per knob:
   bfs_words        64-tree words grown per BFS launch (trees per launch / 64)
-  bfs_group        lanes sharing one vertex in the BFS (the words, or twice that)
+  bfs_group        lanes sharing one vertex in the BFS (one or two per half-word, 0: by the graph)
   score_blocks_sm  blocks per SM of the frustration scorer
   gl_lanes         graphL lanes per row segment (8 -> 32 columns, 16 -> 64, 32 -> 128)
 Choices are cached in JSON per (GPU name, graph shape bucket, K, R), so a
@@ -56,7 +56,8 @@ def _time_family(sb, fam: str, fn, reps: int) -> float:
 def tune(sb, K: int = 1024, R: int | None = None, seed: int = 987654321, reps: int = 2, use_cache: bool = True):
     """Picks the knobs for sampling K trees (and graphL with R start points)
     on the graph loaded in `sb`; returns the chosen values (also applied)."""
-    key = f"{torch.cuda.get_device_name(sb.device)}|{_bucket(sb.n, sb.m)}|K{K}|R{R}"
+    # (entries without "|h" were timed with one lane per word)
+    key = f"{torch.cuda.get_device_name(sb.device)}|{_bucket(sb.n, sb.m)}|K{K}|R{R}|h"
     cache = _load() if use_cache else {}
     if key in cache:
         sb.set_tuning(**cache[key])
@@ -81,12 +82,12 @@ def tune(sb, K: int = 1024, R: int | None = None, seed: int = 987654321, reps: i
     chosen["bfs_words"] = best[1]
     sb.set_tuning(bfs_words=best[1])
 
-    # lanes per vertex group (at least the words of a launch)
-    g0 = 1
-    while g0 < best[1]:
+    # lanes per vertex group: the library's rule (0), one per half-word of a launch, or two
+    g0 = 2
+    while g0 < min(32, 2 * best[1]):
         g0 <<= 1
     best = None
-    for g in sorted({g0, min(32, 2 * g0)}):  # the library widens a group at most twofold
+    for g in sorted({0, g0, min(32, 2 * g0)}):
         sb.set_tuning(bfs_group=g)
         t = _time_family(sb, "bfs", sample, reps)
         if best is None or t < best[0]:

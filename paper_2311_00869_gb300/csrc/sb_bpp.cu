@@ -880,17 +880,20 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
     // A graph too small to fill the SMs that way spreads the trees of a
     // half-word over more lanes, which shortens every lane's run of hashes
     // (1000 vertices, 64 trees: 70 us with 2 lanes per vertex, 43 with 32).  The
-    // knob asks for that width.
+    // knob asks for one lane per half-word or two; a width found for a launch of
+    // more words is not taken over (64 trees on the 2^20 graph: 1.92 ms with 2
+    // lanes, 3.02 with 4, 6.5 for the step with 32).
     int ls = 0;
     const int Gt = (int)c->tune[SB_TUNE_BFS_GROUP];
-    while (G < Gt) {
-        G <<= 1;
-        ls++;
+    const bool asked = Gt == G || Gt == 2 * G;
+    if (asked && Gt > G) {
+        G = Gt;
+        ls = 1;
     }
     // and so does a dense one that fills them a few times over only: its rows
     // take long, and whole warps hash without a queue
     const bool dense = c->n_items < BFS_SPREAD_ITEMS && 2 * c->m >= 16 * c->n;
-    while (Gt == 0 && G < 32 && (dense || c->n_items * slices * G < (int64_t)c->num_sms * BFS_SPREAD_THREADS)) {
+    while (!asked && G < 32 && (dense || c->n_items * slices * G < (int64_t)c->num_sms * BFS_SPREAD_THREADS)) {
         G <<= 1;
         ls++;
     }

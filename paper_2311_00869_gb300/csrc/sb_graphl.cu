@@ -136,8 +136,9 @@ __device__ __forceinline__ float gl_value(const GlArgs& A, float x, float scale_
 // 2.93 for the step below): 11.6 TB/s of gathered rows out of L2, a third of
 // them from DRAM, is what the memory system gives.  Rows that are not 16-byte
 // aligned (R not a multiple of 4) are taken in 32-column pieces, up to four
-// per lane (STRIDED): at 37 columns 2.05 -> 1.26 ms a step.  Traced step on the 2^20 R-MAT graph, 256 columns: 4.58 -> 2.98 ms
-// (and 0.12 for k_gl_count); 64 columns without a trace: 1.47 -> 0.89 ms.
+// per lane (STRIDED): 25 traced steps at 37 columns 53.9 -> 34.0 ms.  Traced
+// step on the 2^20 R-MAT graph, 256 columns: 4.58 -> 2.98 ms (and 0.12 for
+// k_gl_count); 64 columns without a trace: 1.47 -> 0.89 ms.
 template <int VEC, int SL, bool STRIDED, bool STEP, int IB>
 __global__ void __launch_bounds__(GL_THREADS, STRIDED && VEC > 1 ? 4 : GL_ROWS_MIN_BLOCKS) k_gl_rows(GlArgs A)
 {
