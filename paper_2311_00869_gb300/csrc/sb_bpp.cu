@@ -1301,9 +1301,16 @@ extern "C" sb_status sb_batch_steps(sb_ctx* c, uint64_t seed, int64_t tree_begin
     sb_status st = batch_step_enqueue(c);
     if (st == SB_OK && steps > 1) {
         if (use_graph) {
-            const uint64_t key[8] = {seed, (uint64_t)K, (uint64_t)G, c->graph_gen, (uint64_t)bfs_words_per_launch(c),
-                                     (uint64_t)c->tune[SB_TUNE_BFS_GROUP], (uint64_t)c->tune[SB_TUNE_SCORE_BLOCKS_SM],
-                                     (uint64_t)c->tune[SB_TUNE_WAIT_US]};
+            // what the captured launches were made from: arguments, knobs, and the
+            // buffers the step before this one left (any of them may have grown
+            // since the capture, in a call with more trees)
+            auto at = [](const void* p) { return (uint64_t)(uintptr_t)p; };
+            const uint64_t key[SB_BS_KEY] = {seed, (uint64_t)K, (uint64_t)G, c->graph_gen, (uint64_t)bfs_words_per_launch(c),
+                                             (uint64_t)c->tune[SB_TUNE_BFS_GROUP], (uint64_t)c->tune[SB_TUNE_SCORE_BLOCKS_SM],
+                                             (uint64_t)c->tune[SB_TUNE_WAIT_US], (uint64_t)c->tune[SB_TUNE_STALL_TEST],
+                                             at(c->labels), at(c->flipw), at(c->hraw), at(c->hwsum), at(c->hashes),
+                                             at(c->counts), at(c->vis), at(c->fr0), at(c->fr1), at(c->done), at(c->hubnew),
+                                             at(c->hubbest), at(c->sync), at(c->bs_frmin), at(c->bs_fm), at(c->bs_ns)};
             // capture and replay on a private stream ordered after / before
             // the context stream (the legacy default stream cannot be captured)
             if (!c->cap_stream) {

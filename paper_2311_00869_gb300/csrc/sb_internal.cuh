@@ -15,6 +15,7 @@
 #define SB_TREES_MAX (64 * 64)   // trees per sb_sample_trees call
 #define SB_BFS_CHUNK 512         // CSR entries per BFS work item
 #define SB_GL_CHUNK 256          // CSR entries per graphL work item
+#define SB_BS_KEY 25             // words of the captured batch step's key
 #define SB_NEG_BIT 0x80000000u   // sign bit packed into CSR / edge-list ids
 #define SB_ID_MASK 0x7FFFFFFFu
 
@@ -206,7 +207,7 @@ struct sb_ctx {
     int32_t* bs_ns = nullptr;      // G: distinct states of the step
     size_t bs_cap = 0;
     cudaGraphExec_t bs_exec = nullptr;
-    uint64_t bs_exec_key[8] = {0};
+    uint64_t bs_exec_key[SB_BS_KEY] = {0};
     uint64_t graph_gen = 0;        // changes with every loaded graph
 
     // captured descent loop (replayed while its arguments stay the same)
