@@ -1062,9 +1062,7 @@ __global__ void k_fill_i32(int32_t* p, int64_t n, int32_t v)
         p[i] = v;
 }
 
-// Waits for the stream and reports the sampler's error word, and the scorer's
-// when it has just been enqueued (one copy covers both).
-static sb_status check_sync_error(sb_ctx* c, bool scored = false)
+sb_status sb_check_batch(sb_ctx* c, bool scored)
 {
     uint32_t w[23] = {0};  // sync[6 .. 28]
     SB_CHECK_CUDA(c, cudaMemcpyAsync(w, c->sync + 6, sizeof(w), cudaMemcpyDeviceToHost, c->stream));
@@ -1102,7 +1100,7 @@ sb_status sb_batch_begin(sb_ctx* c, uint64_t seed, int64_t tree_begin, int64_t K
     c->tree_begin = tree_begin;
     c->K = K;
     c->W = W;
-    c->counts_valid = false;
+    c->counts_valid = c->batch_checked = false;
     c->batch_in_cloud = false;
     k_batch_begin<<<1, 32, 0, c->stream>>>(c->sync, tree_begin);
     return sb_after_launch(c, "k_batch_begin");
@@ -1349,10 +1347,9 @@ extern "C" sb_status sb_frustration(sb_ctx* c, int32_t* counts_out, uint64_t* ha
     if (!c) return SB_ERR_ARG;
     if (!c->has_batch) return sb_fail(c, SB_ERR_STATE, "no sampled batch");
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
-    const bool score = !c->counts_valid;
-    if (score) SB_TRY(sb_score_enqueue(c));  // behind the sampler; one wait then covers both
-    SB_TRY(check_sync_error(c, score && c->m > 0));
-    c->counts_valid = true;
+    if (!c->counts_valid) SB_TRY(sb_score_enqueue(c));  // behind the sampler; one wait then covers both
+    SB_TRY(sb_check_batch(c, c->m > 0));
+    c->counts_valid = c->batch_checked = true;
     if (c->batch_G > 0) {
         // per graph: K entries, packed graph after graph
         const size_t KP = 64 * (size_t)c->W, K = (size_t)c->K, G = (size_t)c->batch_G;
@@ -1375,7 +1372,7 @@ extern "C" sb_status sb_label(sb_ctx* c, uint64_t* labels_out)
     if (!c || !labels_out) return SB_ERR_ARG;
     if (!c->has_batch) return sb_fail(c, SB_ERR_STATE, "no sampled batch");
     SB_CHECK_CUDA(c, cudaSetDevice(c->device));
-    SB_TRY(check_sync_error(c));
+    SB_TRY(sb_check_batch(c, false));
     int64_t total = c->n * c->W;
     size_t bytes = sizeof(uint64_t) * (size_t)total;
     uint64_t* tmp = (uint64_t*)sb_dalloc(c, bytes);

@@ -139,6 +139,7 @@ struct sb_ctx {
     int32_t* counts = nullptr;    // K
     size_t counts_cap = 0;
     bool counts_valid = false;
+    bool batch_checked = false;   // the device's error words were read after the counts, and clear
     bool batch_in_cloud = false;
     size_t labels_cap = 0;
 
@@ -281,6 +282,9 @@ sb_status sb_radix_sort_u64(sb_ctx* c, uint64_t** keys, uint64_t** alt, int64_t 
 sb_status sb_cloud_insert_batch(sb_ctx* c, int32_t* meta_out);
 sb_status sb_cloud_alloc(sb_ctx* c);
 sb_status sb_score_batch(sb_ctx* c);
+// waits for the stream and reports the sampler's error word, and the scorer's
+// when it has been enqueued (one copy covers both)
+sb_status sb_check_batch(sb_ctx* c, bool scored);
 // sampled-batch storage for trees [tree_begin, tree_begin + K) (labels,
 // canonical flips, counts, hashes), then the canonical flip and state hash
 // once a sampler has written raw labels

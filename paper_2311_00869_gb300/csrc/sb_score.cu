@@ -221,17 +221,12 @@ sb_status sb_score_enqueue(sb_ctx* c)
 }
 
 // counts of the current batch, checked: waits for the launches and reports a
-// tile copy that timed out
+// sampler or a tile copy that gave up (no cloud takes such a batch)
 sb_status sb_score_batch(sb_ctx* c)
 {
-    if (c->counts_valid) return SB_OK;
-    SB_TRY(sb_score_enqueue(c));
-    if (c->m > 0) {
-        uint32_t err = 0;
-        SB_CHECK_CUDA(c, cudaMemcpyAsync(&err, c->sync + 28, sizeof(err), cudaMemcpyDeviceToHost, c->stream));
-        SB_CHECK_CUDA(c, cudaStreamSynchronize(c->stream));
-        if (err) return sb_fail(c, SB_ERR_TIMEOUT, "scorer tile copy timed out");
-    }
-    c->counts_valid = true;
+    if (c->counts_valid && c->batch_checked) return SB_OK;
+    if (!c->counts_valid) SB_TRY(sb_score_enqueue(c));
+    SB_TRY(sb_check_batch(c, c->m > 0));
+    c->counts_valid = c->batch_checked = true;
     return SB_OK;
 }
