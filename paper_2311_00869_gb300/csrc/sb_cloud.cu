@@ -787,7 +787,8 @@ extern "C" sb_status sb_cloud_switch(sb_ctx* c, int64_t idx, uint64_t* edge_bits
 // the leader bit for bit over the graph's vertices, and a tree that differs
 // starts its own state (matched, if possible, against the earlier differing
 // trees of the run).  Output per graph: number of states, min S, and the
-// states in order of first appearance.
+// states in order of first appearance (first trees count from tree0, the batch's
+// first tree on the host: after sb_batch_steps the device's copy has moved on).
 #define BC_MAXK 1024
 #define BC_THREADS 256
 
@@ -807,7 +808,7 @@ __device__ bool bc_same(const uint64_t* lab, int W, const uint64_t* flip, int64_
 
 __global__ void __launch_bounds__(BC_THREADS)
     k_batch_cloud(const uint64_t* __restrict__ hashes, const int32_t* __restrict__ counts, int64_t KP, int K,
-                  const int64_t* __restrict__ tree0p, const uint64_t* __restrict__ lab, int W,
+                  int64_t tree0, const uint64_t* __restrict__ lab, int W,
                   const uint64_t* __restrict__ flipw,
                   const int32_t* __restrict__ voff, int32_t* __restrict__ nstates_out, int32_t* __restrict__ frmin_out,
                   sb_cloud_entry* __restrict__ entries)
@@ -920,7 +921,7 @@ __global__ void __launch_bounds__(BC_THREADS)
                 e.hash = hashes[g * KP + t];
                 e.S = counts[g * KP + t];
                 e.count = cnt[t];
-                e.first_tree = *tree0p + t;
+                e.first_tree = tree0 + t;
                 entries[g * (int64_t)K + rank[t]] = e;
             }
     if (tid == 0) {
@@ -946,8 +947,8 @@ extern "C" sb_status sb_batch_cloud(sb_ctx* c, int32_t* n_states_out, int32_t* f
     if (st == SB_OK) {
         SbProf prof(c, SB_PROF_CLOUD);
         k_batch_cloud<<<(unsigned)G, BC_THREADS, 0, c->stream>>>(c->hashes, c->counts, 64 * (int64_t)c->W, (int)c->K,
-                                                                sb_tree0_ptr(c->sync), c->labels, c->W, c->flipw,
-                                                                c->b_voff, ns, fm, ent);
+                                                                c->tree_begin, c->labels, c->W, c->flipw, c->b_voff,
+                                                                ns, fm, ent);
         st = sb_after_launch(c, "k_batch_cloud");
     }
     if (st == SB_OK) st = sb_copy_out(c, n_states_out, ns, sizeof(int32_t) * (size_t)G);
@@ -966,8 +967,7 @@ sb_status sb_batch_cloud_enqueue(sb_ctx* c, int32_t* n_states, int32_t* fr_min)
 {
     SbProf prof(c, SB_PROF_CLOUD);
     k_batch_cloud<<<(unsigned)c->batch_G, BC_THREADS, 0, c->stream>>>(c->hashes, c->counts, 64 * (int64_t)c->W,
-                                                                     (int)c->K, sb_tree0_ptr(c->sync), c->labels,
-                                                                     c->W, c->flipw, c->b_voff, n_states, fr_min,
-                                                                     nullptr);
+                                                                     (int)c->K, 0, c->labels, c->W, c->flipw,
+                                                                     c->b_voff, n_states, fr_min, nullptr);
     return sb_after_launch(c, "k_batch_cloud");
 }

@@ -64,3 +64,27 @@ def test_capture_during_a_barrier_test_is_not_replayed():
         _check(sb, refs, 3, 0, 64, 3)
     finally:
         sb.close()
+
+
+@pytest.mark.parametrize("use_graph", [True, False])
+def test_clouds_after_steps_are_the_last_steps(use_graph):
+    """The batch that sb_batch_steps leaves is the last step's: the per-graph
+    clouds taken from it name that step's trees."""
+    import paper_2311_00869_gb300 as P
+
+    graphs = _graphs()
+    K, steps, t0 = 64, 3, 20
+    sb = P.SignedBal(0)
+    try:
+        sb.load_batch(graphs)
+        sb.batch_steps(5, t0, K, steps, use_graph=use_graph)
+        sb.sync()
+        cl = sb.batch_cloud()
+        for g, r in enumerate(O.clean_graph(*x) for x in graphs):
+            ref = O.sample(r, 5, t0 + (steps - 1) * K, K)
+            rc = O.cloud(ref["labels"], ref["counts"], t0=t0 + (steps - 1) * K)
+            assert cl["n_states"][g] == rc["S"].shape[0], g
+            for k, o in (("first_tree", "first_tree"), ("count", "count"), ("S", "S"), ("hash", "H")):
+                assert np.array_equal(cl["entries"][g][k], rc[o]), (g, k)
+    finally:
+        sb.close()
