@@ -202,22 +202,32 @@ __global__ void k_emit_edges(const uint64_t* __restrict__ keys, int64_t m, int n
 }
 
 // The edges are sorted by u and the lower keys by v, so the first position of
-// every vertex in either follows from where neighbours differ (no counting
-// atomics, which the hubs would serialise):
+// every vertex in either is where its rows start (no counting atomics, which
+// the hubs would serialise):
 //   ufirst[x], lfirst[x] = first edge with u >= x, first key with v >= x
 // (n + 1 entries).  A row is its lower neighbours, then its upper ones, so
 //   rowptr[x] = ufirst[x] + lfirst[x],
 //   entry of edge i in row u   = lfirst[u + 1] + i,
 //   entry of key p in row v    = ufirst[v] + p.
+// Every vertex finds its two by binary search: filling the gap between two
+// neighbouring ends from there instead is one thread's loop over all of it, and
+// ids that are never a smaller (or larger) end, the items of a graph that
+// numbers its users first, leave a gap as long as their number (2 M users, 8 M
+// items, 32 M edges: 26.7 ms by gaps, 0.33 ms by searches; with permuted ids the
+// search takes 0.32 ms and a load as long as with gaps).
 __global__ void k_first(const int2* __restrict__ edges, const uint64_t* __restrict__ lkeys, int64_t m, int64_t n, int nb2,
                         int32_t* __restrict__ ufirst, int32_t* __restrict__ lfirst)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= m; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t a = i > 0 ? edges[i - 1].x : -1, b = i < m ? edges[i].x : n;
-        for (int64_t x = a + 1; x <= b; x++) ufirst[x] = (int32_t)i;
-        a = i > 0 ? (int64_t)(lkeys[i - 1] >> (nb2 + 1)) : -1;
-        b = i < m ? (int64_t)(lkeys[i] >> (nb2 + 1)) : n;
-        for (int64_t x = a + 1; x <= b; x++) lfirst[x] = (int32_t)i;
+    uint32_t top = 0;  // largest power of two <= m
+    if (m > 0) top = 1u << (31 - __clz((int)m));
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t a = 0, b = 0;  // this many are below x, as far as known
+        for (uint32_t step = top; step; step >>= 1) {
+            if (a + step <= m && edges[a + step - 1].x < x) a += step;
+            if (b + step <= m && (int64_t)(lkeys[b + step - 1] >> (nb2 + 1)) < x) b += step;
+        }
+        ufirst[x] = (int32_t)a;
+        lfirst[x] = (int32_t)b;
     }
 }
 
@@ -716,10 +726,10 @@ static sb_status load_graph_impl(sb_ctx* c, int64_t n, int64_t m, const int32_t*
         return sb_fail(c, SB_ERR_OOM, "graph storage");
     k_emit_edges<<<gm1, 256, 0, c->stream>>>(ukeys, m1, nb, ekeep, epos, newid, nb2, c->edges, lkeys);
     SB_TRY(sb_after_launch(c, "k_emit_edges"));
-    unsigned gm2 = grid_for(c, m2 + 1), gn1 = grid_for(c, n1 + 1);
+    unsigned gm2 = grid_for(c, m2), gn1 = grid_for(c, n1 + 1);
     // by v alone: the keys come in (u, v) order and the sort is stable
     SB_TRY(sb_radix_sort_u64(c, &lkeys, &alt, m2, nb2 + 1, 2 * nb2 + 1));
-    k_first<<<gm2, 256, 0, c->stream>>>(c->edges, lkeys, m2, n1, nb2, ufirst, lfirst);
+    k_first<<<gn1, 256, 0, c->stream>>>(c->edges, lkeys, m2, n1, nb2, ufirst, lfirst);
     SB_TRY(sb_after_launch(c, "k_first"));
     k_rowptr<<<gn1, 256, 0, c->stream>>>(ufirst, lfirst, n1, c->rowptr, deg);
     SB_TRY(sb_after_launch(c, "k_rowptr"));
