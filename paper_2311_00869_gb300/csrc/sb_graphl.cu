@@ -121,9 +121,16 @@ __device__ __forceinline__ float gl_value(const GlArgs& A, float x, float scale_
 // vertex order) rarely crosses a graph of a batch.  A graph too small for
 // every sub-warp to get GL_ROWS_PER_SUB rows takes them one at a time: with
 // blocks of 16, 1000 rows kept 63 of 4864 warps busy, each with 16 rows in
-// turn (33.7 us a descent step at 5 columns, now 6.4).
+// turn (33.7 us a descent step at 5 columns, now 6.4).  Batches of graphs take
+// blocks earlier, and a step over a batch always: a sub-warp's column maxima go
+// to its graph's accumulators whenever the graph changes, and rows one at a time
+// change it at every row (256 graphs of 3000 vertices, 32 columns: 627 us a step,
+// 155 in blocks).  Gradient over 4096 graphs of 50 vertices, one by one against
+// blocks: 39 / 45 us at 8 rows per sub-warp (32 columns), 72 / 58 at 16 (64),
+// 193 / 138 at 32 (256).
 #define GL_ITEM_BLOCK 16
 #define GL_ROWS_PER_SUB 32
+#define GL_ROWS_PER_SUB_BATCH 12
 //
 // What bounds it: the gathers.  Long-scoreboard stalls led at half the warps
 // resident, so a lane keeps GL_INFLIGHT neighbour rows in flight (the last,
@@ -772,7 +779,8 @@ static sb_status gl_rows_launch(sb_ctx* c, GlArgs& A)
     A.vec_out = (((uintptr_t)A.gout_rows | (uintptr_t)A.upstream) & 15) == 0;
     const int subs = GL_THREADS / (vec4 && lanes != 32 ? (lanes == 16 ? 16 : 8) : 32);
     const int64_t rows = A.n_items - A.n_split_items;
-    const bool small = rows < (int64_t)c->num_sms * GL_ROWS_MIN_BLOCKS * subs * GL_ROWS_PER_SUB;
+    const int64_t fill = (int64_t)c->num_sms * GL_ROWS_MIN_BLOCKS * subs;
+    const bool small = !(STEP && A.vgid) && rows < fill * (A.vgid ? GL_ROWS_PER_SUB_BATCH : GL_ROWS_PER_SUB);
     const void* fn = small ? gl_rows_kernel<STEP, 1>(vec4, lanes, A.R) : gl_rows_kernel<STEP, GL_ITEM_BLOCK>(vec4, lanes, A.R);
     size_t smem = STEP ? sizeof(uint32_t) * (size_t)A.R : 0;
     if (smem > 48 * 1024) SB_CHECK_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
