@@ -114,30 +114,37 @@ struct ScoreAcc {
                 if (val) atomicAdd(dst + 64 * lane + t, val);
             }
         } else {
-            constexpr uint32_t M = G == 1 ? 0xFFFFFFFFu : G == 2 ? 0x55555555u : G == 4 ? 0x11111111u
-                                 : G == 8 ? 0x01010101u : 0x00010001u;  // lanes of word 0
             uint32_t lo[G], hi[G];
-#pragma unroll
-            for (int w = 0; w < G; w++) lo[w] = hi[w] = 0;
-            auto add = [&](uint64_t x, int shift) {
-                if (!__any_sync(0xffffffffu, x != 0)) return;
-                const uint32_t a = warp_transpose32((uint32_t)x, lane), b = warp_transpose32((uint32_t)(x >> 32), lane);
-#pragma unroll
-                for (int w = 0; w < G; w++) {
-                    lo[w] += (uint32_t)__popc(a & (M << w)) << shift;
-                    hi[w] += (uint32_t)__popc(b & (M << w)) << shift;
-                }
-            };
-            add(ones, 0);
-            add(twos, 1);
-            add(fours, 2);
-#pragma unroll
-            for (int b = 0; b < SC_PLANES; b++) add(P[b], 3 + b);
+            sum_warp<G>(lo, hi);
 #pragma unroll
             for (int w = 0; w < G; w++) {
                 if (lo[w]) atomicAdd(dst + 64 * w + lane, lo[w]);
                 if (hi[w]) atomicAdd(dst + 64 * w + 32 + lane, hi[w]);
             }
         }
+    }
+    // the warp's counts of streams `lane` and `lane + 32` of word w in lo[w], hi[w]
+    template <int G>
+    __device__ __forceinline__ void sum_warp(uint32_t* lo, uint32_t* hi) const
+    {
+        constexpr uint32_t M = G == 1 ? 0xFFFFFFFFu : G == 2 ? 0x55555555u : G == 4 ? 0x11111111u
+                             : G == 8 ? 0x01010101u : 0x00010001u;  // lanes of word 0
+        const unsigned lane = threadIdx.x & 31u;
+#pragma unroll
+        for (int w = 0; w < G; w++) lo[w] = hi[w] = 0;
+        auto add = [&](uint64_t x, int shift) {
+            if (!__any_sync(0xffffffffu, x != 0)) return;
+            const uint32_t a = warp_transpose32((uint32_t)x, lane), b = warp_transpose32((uint32_t)(x >> 32), lane);
+#pragma unroll
+            for (int w = 0; w < G; w++) {
+                lo[w] += (uint32_t)__popc(a & (M << w)) << shift;
+                hi[w] += (uint32_t)__popc(b & (M << w)) << shift;
+            }
+        };
+        add(ones, 0);
+        add(twos, 1);
+        add(fours, 2);
+#pragma unroll
+        for (int b = 0; b < SC_PLANES; b++) add(P[b], 3 + b);
     }
 };

@@ -368,35 +368,30 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_signs(const float* __restrict
     }
 }
 
-// Frustrated edges per column from the sign words (vertical counters, as in
-// the scorer): a group of G lanes takes an edge, lane = 64 columns, a warp a
-// contiguous range of the edges.  counts[graph * KS + slot].  Latency bounds
-// it: 490 us per pass (16.8 M edges, 256 columns) with a check before every
-// load, 264 without, 115 with the next batch's edges loaded ahead and the
-// counters flushed by transposes.
-template <int G, bool SEG>
+// Frustrated edges per column of one graph from the sign words (vertical
+// counters, as in the scorer): a group of G lanes takes an edge, lane = 64
+// columns, a warp a contiguous range of the edges.  Latency bounds it: 490 us per
+// pass (16.8 M edges, 256 columns) with a check before every load, 264 without,
+// 115 with the next batch's edges loaded ahead and the counters flushed by
+// transposes.
+template <int G>
 __global__ void __launch_bounds__(GL_THREADS) k_gl_count(const int2* __restrict__ edges, int64_t m,
                                                          const uint64_t* __restrict__ signs, int W,
-                                                         const int32_t* __restrict__ vgid, int64_t KS,
                                                          uint32_t* __restrict__ counts)
 {
-    __shared__ uint32_t scnt[64 * G];  // block counts (one graph)
+    __shared__ uint32_t scnt[64 * G];
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), grp = lane / G;
     const int word = blockIdx.y * 32 + gl;
     const bool act = word < W;
     constexpr int NG = 32 / G;
-    if (!SEG) {
-        for (int i = threadIdx.x; i < 64 * G; i += GL_THREADS) scnt[i] = 0;
-        __syncthreads();
-    }
+    for (int i = threadIdx.x; i < 64 * G; i += GL_THREADS) scnt[i] = 0;
+    __syncthreads();
     const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32);
     const int64_t per = sb_cdiv(sb_cdiv(m, 8 * NG), warps) * (8 * NG);
     const int64_t wid = (int64_t)blockIdx.x * (GL_THREADS / 32) + (threadIdx.x >> 5);
     const int64_t e1 = min(m, (wid + 1) * per);
-    uint32_t* const dst = SEG ? counts + 64 * word : scnt + 64 * gl;
     ScoreAcc acc;
     acc.reset();
-    int64_t gcur = -1;
     int2 nx[8];
     auto load = [&](int64_t e) {
 #pragma unroll
@@ -419,28 +414,97 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_count(const int2* __restrict_
             for (int k = 0; k < 8; k++)
                 x[k] = signs[(int64_t)ed[k].x * W + word] ^ signs[(int64_t)((uint32_t)ed[k].y & SB_ID_MASK) * W + word] ^
                        (uint64_t)(int64_t)(ed[k].y >> 31);  // 0 past the end: an edge (0, 0)
-            if (SEG) {
-                int32_t gk[8];
-                uint32_t rem = 0;
+            acc.add8(x);
+            if (acc.nb == SC_FLUSH) acc.flush(scnt + 64 * gl);
+        }
+    acc.template flush_warp<G>(scnt);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 64 * G; i += GL_THREADS)
+        if (scnt[i]) atomicAdd(counts + (int64_t)blockIdx.y * 2048 + i, scnt[i]);
+}
+
+// The same for a batch: counts[graph * KS + slot].  A warp takes a contiguous range of
+// the edges (graph after graph) and 64 columns (blockIdx.y), a lane an edge.  256
+// edges of one graph go into vertical counters; where graphs change, 32 edges at a
+// time are transposed and each graph's share is counted under its lanes' mask, so
+// that a graph costs its own edges and one flush.  With vertical counters alone
+// every lane flushed 64 counters whenever it met another graph (20,000 graphs of
+// 9 edges, 5 columns: 166 us a pass, 6 here).
+__global__ void __launch_bounds__(GL_THREADS) k_gl_count_graphs(const int2* __restrict__ edges, int64_t m,
+                                                                const int32_t* __restrict__ vgid,
+                                                                const uint64_t* __restrict__ signs, int W, int64_t KS,
+                                                                uint32_t* __restrict__ counts)
+{
+    const int lane = threadIdx.x & 31, word = blockIdx.y;
+    const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32);
+    const int64_t per = sb_cdiv(m, 32 * warps) * 32;
+    const int64_t wid = (int64_t)blockIdx.x * (GL_THREADS / 32) + (threadIdx.x >> 5);
+    const int64_t e1 = min(m, (wid + 1) * per);
+    ScoreAcc acc;
+    acc.reset();
+    int64_t gcur = -1;
+    uint32_t lo = 0, hi = 0;  // of graph gcur, this lane's columns
+    auto sum = [&]() {
+        if (!acc.nb) return;
+        uint32_t l, h;
+        acc.template sum_warp<1>(&l, &h);
+        lo += l;
+        hi += h;
+        acc.reset();
+    };
+    auto turn = [&](int64_t g) {  // to graph g
+        if (g == gcur) return;
+        if (gcur >= 0) {
+            sum();
+            uint32_t* const dst = counts + gcur * KS + 64 * word;
+            if (lo) atomicAdd(dst + lane, lo);
+            if (hi) atomicAdd(dst + 32 + lane, hi);
+        }
+        gcur = g;
+        lo = hi = 0;
+    };
+    for (int64_t e = wid * per; e < e1; e += 256) {
+        int2 ed[8];
+        int32_t gk[8];
+        uint64_t x[8];
 #pragma unroll
-                for (int k = 0; k < 8; k++) {
-                    gk[k] = vgid[ed[k].x];
-                    rem |= (e + k * NG < e1 ? 1u : 0u) << k;
-                }
-                acc.add8_runs(x, gk, rem, gcur, dst, KS);
-            } else {
-                acc.add8(x);
-                if (acc.nb == SC_FLUSH) acc.flush(dst);
+        for (int k = 0; k < 8; k++) {
+            ed[k] = make_int2(-1, 0);
+            if (e + 32 * k + lane < e1) ed[k] = __ldg(edges + e + 32 * k + lane);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            gk[k] = -1;
+            x[k] = 0;
+            if (ed[k].x >= 0) {
+                gk[k] = vgid[ed[k].x];
+                x[k] = signs[(int64_t)ed[k].x * W + word] ^ signs[(int64_t)((uint32_t)ed[k].y & SB_ID_MASK) * W + word] ^
+                       (uint64_t)(int64_t)(ed[k].y >> 31);
             }
         }
-    if (SEG) {
-        if (act && gcur >= 0) acc.flush(dst + gcur * KS);
-    } else {
-        acc.template flush_warp<G>(scnt);
-        __syncthreads();
-        for (int i = threadIdx.x; i < 64 * G; i += GL_THREADS)
-            if (scnt[i]) atomicAdd(counts + (int64_t)blockIdx.y * 2048 + i, scnt[i]);
+        const int32_t g0 = __shfl_sync(0xffffffffu, gk[0], 0);
+        if (g0 == __shfl_sync(0xffffffffu, gk[7], 31)) {  // 256 edges of one graph
+            turn(g0);
+            acc.add8(x);
+            if (acc.nb == SC_FLUSH) sum();
+            continue;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            uint32_t rem = __ballot_sync(0xffffffffu, gk[k] >= 0);
+            if (!rem) break;
+            const uint32_t a = warp_transpose32((uint32_t)x[k], lane), b = warp_transpose32((uint32_t)(x[k] >> 32), lane);
+            while (rem) {
+                const int32_t g = __shfl_sync(0xffffffffu, gk[k], __ffs((int)rem) - 1);
+                const uint32_t mask = __ballot_sync(0xffffffffu, gk[k] == g);
+                turn(g);
+                lo += (uint32_t)__popc(a & mask);
+                hi += (uint32_t)__popc(b & mask);
+                rem &= ~mask;
+            }
+        }
     }
+    turn(-1);
 }
 
 // Alg. 2 rounding: bit per edge and column, from the sign words: a warp takes
@@ -703,32 +767,35 @@ static sb_status gl_signs_launch(sb_ctx* c, const float* gamma, int R, uint32_t*
     return sb_after_launch(c, "k_gl_signs");
 }
 
-template <bool SEG>
 static const void* gl_count_kernel(int W)
 {
-    return W > 16  ? (const void*)k_gl_count<32, SEG>
-           : W > 8 ? (const void*)k_gl_count<16, SEG>
-           : W > 4 ? (const void*)k_gl_count<8, SEG>
-           : W > 2 ? (const void*)k_gl_count<4, SEG>
-           : W > 1 ? (const void*)k_gl_count<2, SEG>
-                   : (const void*)k_gl_count<1, SEG>;
+    return W > 16  ? (const void*)k_gl_count<32>
+           : W > 8 ? (const void*)k_gl_count<16>
+           : W > 4 ? (const void*)k_gl_count<8>
+           : W > 2 ? (const void*)k_gl_count<4>
+           : W > 1 ? (const void*)k_gl_count<2>
+                   : (const void*)k_gl_count<1>;
 }
 
 // adds the frustrated edges of every column to `counts` (gl_slots per graph)
 static sb_status gl_count_launch(sb_ctx* c, const uint32_t* signs, int R, uint32_t* counts)
 {
     if (c->m == 0) return SB_OK;
-    const bool seg = c->batch_G > 0;
     int W = gl_sign_words(R) / 2;
-    const void* fn = seg ? gl_count_kernel<true>(W) : gl_count_kernel<false>(W);
     const int2* edges = c->sc_edges;  // first endpoints repeat over a run of edges, second ones are often hubs
-    int64_t m = c->m, KS = gl_slots(R);
-    const int32_t* vgid = c->vgid;
+    int64_t m = c->m;
+    if (c->batch_G > 0) {  // (the scorer's edges lie graph after graph, as the sorted ones)
+        // a warp takes at least 64 edges
+        const unsigned bx = (unsigned)std::max<int64_t>(
+            1, std::min<int64_t>(sb_cdiv(m, 64 * (GL_THREADS / 32)), sb_cdiv((int64_t)c->num_sms * 8, std::min(W, 8))));
+        k_gl_count_graphs<<<dim3(bx, (unsigned)W), GL_THREADS, 0, c->stream>>>(edges, m, c->vgid, (const uint64_t*)signs, W, gl_slots(R), counts);
+        return sb_after_launch(c, "k_gl_count_graphs");
+    }
     // a warp takes at least 4 batches of 8 edges per group
     const int64_t batches = sb_cdiv(m * std::min(W, 32), 8 * 32 * 4 * (GL_THREADS / 32));
     const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(batches, (int64_t)c->num_sms * 4));
-    void* args[] = {(void*)&edges, &m, (void*)&signs, &W, (void*)&vgid, &KS, &counts};
-    SB_CHECK_CUDA(c, cudaLaunchKernel(fn, dim3(bx, (unsigned)sb_cdiv(W, 32)), dim3(GL_THREADS), args, 0, c->stream));
+    void* args[] = {(void*)&edges, &m, (void*)&signs, &W, &counts};
+    SB_CHECK_CUDA(c, cudaLaunchKernel(gl_count_kernel(W), dim3(bx, (unsigned)sb_cdiv(W, 32)), dim3(GL_THREADS), args, 0, c->stream));
     return sb_after_launch(c, "k_gl_count");
 }
 

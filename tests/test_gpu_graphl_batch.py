@@ -1,6 +1,7 @@
 """graphL over batches of graphs: discrete losses, flips and traces of every
 graph equal the oracle's for that graph alone, from single edges to graphs of
-many counted batches, and a step's column maxima do not make it slow."""
+many counted batches, and neither many small graphs nor a step's column maxima
+make a descent slow."""
 import time
 
 import numpy as np
@@ -88,5 +89,21 @@ def test_steps_over_a_batch_cost_about_a_gradient():
         gout, out = torch.ones(256 * 32, device="cuda"), torch.empty_like(gam)
         step = _ms(lambda: sb.graphL_descent(gam, 0.05, 20, out=out)) / 20
         assert step <= 2.5 * _ms(lambda: [sb.graphL_bwd(gam, gout) for _ in range(20)]) / 20
+    finally:
+        sb.close()
+
+
+def test_traces_of_many_small_graphs_cost_little():
+    """20,000 graphs of 12 vertices: a traced descent takes at most twice an
+    untraced one (3.9 times with 64 counters flushed per lane and graph)."""
+    import paper_2311_00869_gb300 as P
+
+    sb = P.SignedBal(0)
+    try:
+        sb.load_batch(_uniform(20000, 12, 4, seed=3))
+        gam = torch.rand((sb.n, 5), device="cuda") * 2 - 1
+        out = torch.empty_like(gam)
+        plain = _ms(lambda: sb.graphL_descent(gam, 0.05, 20, out=out))
+        assert _ms(lambda: sb.graphL_descent(gam, 0.05, 20, trace=True, out=out)) <= 2.0 * plain
     finally:
         sb.close()
