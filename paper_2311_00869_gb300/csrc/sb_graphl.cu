@@ -34,7 +34,7 @@ struct GlArgs {
     const float* upstream; // GRAD: gout[G x R] (G = 1 for one graph)
     const float* scale;    // STEP: input scale per (graph, column), a power of two
     float half_alpha;      // STEP: alpha / 2
-    uint32_t* signs;       // STEP: sign words of the output (see sign_slot), nullable
+    uint32_t* signs;       // STEP: sign words of the output (see sign_col), nullable
     int sign_words;        // 32-bit sign words per vertex (even)
     bool vec_out;          // output (and upstream) rows are 16-byte aligned
     uint32_t* colmax;      // STEP: max |G_out| bits per (graph, column)
@@ -50,13 +50,16 @@ __device__ __forceinline__ uint32_t is_neg(float x) { return __float_as_uint(x) 
 // Sign words: bit of column r of G in word r / 32 of a vertex's sign words, 1
 // for theta = -1.  When R is a multiple of 4 a lane of the row kernel holds
 // four adjacent columns, so the word's bits are ordered by (r % 4, r / 4 % 8):
-// byte k holds the lanes' k-th columns, one ballot each.
-__host__ __device__ __forceinline__ int sign_slot(int r, bool quad)
-{
-    return quad ? (r & ~31) + 8 * (r & 3) + ((r & 31) >> 2) : r;
-}
+// byte k holds the lanes' k-th columns, one ballot each.  (Bits of columns past R
+// are 0; a count over edges of such a bit means nothing.)
 // column (of 32) at bit j
 __device__ __forceinline__ int sign_col(int j, bool quad) { return quad ? 4 * (j & 7) + (j >> 3) : j; }
+// adds a count of bit j of the 32-column block `blk` to its column
+__device__ __forceinline__ void add_count(int32_t* F, int R, int blk, int j, uint32_t x)
+{
+    const int r = 32 * blk + sign_col(j, R % 4 == 0);
+    if (x && r < R) atomicAdd(F + r, (int32_t)x);
+}
 // sign word of a warp whose lane c holds column c of 32
 __device__ __forceinline__ uint32_t sign_word(bool neg, bool quad)
 {
@@ -353,18 +356,38 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_combine(GlArgs A, const int32
     }
 }
 
-// Sign words of a whole matrix: a warp takes 32 columns of one vertex.
+// Sign words of a whole matrix: a warp takes 32 columns of one vertex at a time,
+// eight such words loaded together (one by one: 44 us at n = 100,000 and 130
+// columns, 24 so).  Clears `clear` for the counts that follow.
 __global__ void __launch_bounds__(GL_THREADS) k_gl_signs(const float* __restrict__ g, int64_t n, int R,
-                                                         uint32_t* __restrict__ signs, int sign_words)
+                                                         uint32_t* __restrict__ signs, int sign_words,
+                                                         int32_t* __restrict__ clear, int64_t nclear)
 {
-    const int lane = threadIdx.x & 31, nb = (R + 31) / 32;
+    const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32);
-    for (int64_t x = ((int64_t)blockIdx.x * GL_THREADS + threadIdx.x) >> 5; x < n * sign_words; x += warps) {
-        const int64_t v = x / sign_words;
-        const int blk = (int)(x - v * sign_words), r = 32 * blk + lane;
-        uint32_t w = 0;
-        if (blk < nb) w = sign_word(r < R && is_neg(g[v * R + r]), R % 4 == 0);
-        if (lane == 0) signs[x] = w;
+    const int64_t t0 = (int64_t)blockIdx.x * GL_THREADS + threadIdx.x;
+    for (int64_t i = t0; i < nclear; i += 32 * warps) clear[i] = 0;
+    for (int64_t x = (t0 >> 5) * 8; x < n * sign_words; x += 8 * warps) {
+        int64_t v = x / sign_words;
+        int blk = (int)(x - v * sign_words);
+        float y[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const int r = 32 * blk + lane;
+            y[i] = 0.f;
+            if (v < n && r < R) y[i] = g[v * R + r];
+            if (++blk == sign_words) {
+                blk = 0;
+                v++;
+            }
+        }
+        uint32_t mine = 0;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const uint32_t w = sign_word(is_neg(y[i]), R % 4 == 0);
+            if (lane == i) mine = w;
+        }
+        if (lane < 8 && x + lane < n * sign_words) signs[x + lane] = mine;
     }
 }
 
@@ -376,8 +399,8 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_signs(const float* __restrict
 // transposes.
 template <int G>
 __global__ void __launch_bounds__(GL_THREADS) k_gl_count(const int2* __restrict__ edges, int64_t m,
-                                                         const uint64_t* __restrict__ signs, int W,
-                                                         uint32_t* __restrict__ counts)
+                                                         const uint64_t* __restrict__ signs, int W, int R,
+                                                         int32_t* __restrict__ F)
 {
     __shared__ uint32_t scnt[64 * G];
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), grp = lane / G;
@@ -419,11 +442,10 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_count(const int2* __restrict_
         }
     acc.template flush_warp<G>(scnt);
     __syncthreads();
-    for (int i = threadIdx.x; i < 64 * G; i += GL_THREADS)
-        if (scnt[i]) atomicAdd(counts + (int64_t)blockIdx.y * 2048 + i, scnt[i]);
+    for (int i = threadIdx.x; i < 64 * G; i += GL_THREADS) add_count(F, R, blockIdx.y * 64 + i / 32, i & 31, scnt[i]);
 }
 
-// The same for a batch: counts[graph * KS + slot].  A warp takes a contiguous range of
+// The same for a batch: F[graph * R + column].  A warp takes a contiguous range of
 // the edges (graph after graph) and 64 columns (blockIdx.y), a lane an edge.  256
 // edges of one graph go into vertical counters; where graphs change, 32 edges at a
 // time are transposed and each graph's share is counted under its lanes' mask, so
@@ -432,8 +454,8 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_count(const int2* __restrict_
 // 9 edges, 5 columns: 166 us a pass, 6 here).
 __global__ void __launch_bounds__(GL_THREADS) k_gl_count_graphs(const int2* __restrict__ edges, int64_t m,
                                                                 const int32_t* __restrict__ vgid,
-                                                                const uint64_t* __restrict__ signs, int W, int64_t KS,
-                                                                uint32_t* __restrict__ counts)
+                                                                const uint64_t* __restrict__ signs, int W, int R,
+                                                                int32_t* __restrict__ F)
 {
     const int lane = threadIdx.x & 31, word = blockIdx.y;
     const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32);
@@ -456,9 +478,8 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_count_graphs(const int2* __re
         if (g == gcur) return;
         if (gcur >= 0) {
             sum();
-            uint32_t* const dst = counts + gcur * KS + 64 * word;
-            if (lo) atomicAdd(dst + lane, lo);
-            if (hi) atomicAdd(dst + 32 + lane, hi);
+            add_count(F + gcur * R, R, 2 * word, lane, lo);
+            add_count(F + gcur * R, R, 2 * word + 1, lane, hi);
         }
         gcur = g;
         lo = hi = 0;
@@ -509,19 +530,21 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_count_graphs(const int2* __re
 
 // Alg. 2 rounding: bit per edge and column, from the sign words: a warp takes
 // 4 words of 64 edges and 32 columns, lane = edge, and two 32 x 32 bit
-// transposes per word give lane j the edges of the column at bit j.
+// transposes per word give lane j the edges of the column at bit j.  For one
+// graph it also counts them into F (nullable): a warp keeps its columns, since
+// the launch's warps are a multiple of the column blocks.
 __global__ void __launch_bounds__(GL_THREADS) k_gl_flips(const int2* __restrict__ edges, int64_t m,
                                                          const uint32_t* __restrict__ signs, int sign_words, int R,
-                                                         uint64_t* __restrict__ flips)
+                                                         uint64_t* __restrict__ flips, int32_t* __restrict__ F)
 {
     const int lane = threadIdx.x & 31, nb = (R + 31) / 32;
-    const bool quad = R % 4 == 0;
     const int64_t nw = sb_cdiv(m, 64), nq = sb_cdiv(nw, 4);
-    const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32);
-    for (int64_t x = ((int64_t)blockIdx.x * GL_THREADS + threadIdx.x) >> 5; x < nq * nb; x += warps) {
-        const int64_t wq = x / nb;
-        const int blk = (int)(x - wq * nb);
-        const int r = 32 * blk + sign_col(lane, quad);
+    const int64_t rows = (int64_t)gridDim.x * (GL_THREADS / 32) / nb;
+    const int64_t wid = ((int64_t)blockIdx.x * GL_THREADS + threadIdx.x) >> 5;
+    const int blk = (int)(wid % nb);
+    const int r = 32 * blk + sign_col(lane, R % 4 == 0);
+    uint32_t count = 0;
+    for (int64_t wq = wid / nb; wq < nq; wq += rows) {
 #pragma unroll
         for (int i = 0; i < 4; i++) {
             const int64_t w = 4 * wq + i;
@@ -537,22 +560,18 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_flips(const int2* __restrict_
                         signs[(int64_t)((uint32_t)ed.y & SB_ID_MASK) * sign_words + blk] ^ (uint32_t)(ed.y >> 31);
                 }
                 half[h] = warp_transpose32(f, lane);
+                count += (uint32_t)__popc(half[h]);
             }
             if (r < R) flips[(int64_t)r * nw + w] = ((uint64_t)half[1] << 32) | half[0];
         }
     }
+    if (F && r < R && count) atomicAdd(F + r, (int32_t)count);
 }
 
-// per-(graph, column) renorm decision and discrete-loss trace after one step
-__global__ void k_gl_step_final(int64_t GR, int R, int64_t KS, uint32_t* colmax, uint32_t* counts,
-                                int32_t* F_trace_row, float* scale, int32_t* exps, int renorm_log2)
+// per-(graph, column) renorm decision after one step
+__global__ void k_gl_step_final(int64_t GR, uint32_t* colmax, float* scale, int32_t* exps, int renorm_log2)
 {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < GR; r += (int64_t)gridDim.x * blockDim.x) {
-        if (F_trace_row) {
-            uint32_t* f = counts + r / R * KS + sign_slot((int)(r % R), R % 4 == 0);
-            F_trace_row[r] = (int32_t)*f;
-            *f = 0;
-        }
         const float mx = __uint_as_float(colmax[r]);
         colmax[r] = 0;
         float sc = 1.0f;
@@ -571,26 +590,36 @@ __global__ void k_gl_fill(float* p, int64_t n, float v)
 
 // Pending power-of-two scale of the last step, and the sign words (nullable)
 // of what it changes (a scaled value can underflow to zero): a warp takes 32
-// columns of one vertex, and columns without a pending scale cost one read of
-// the scale.
+// columns of four vertices at a time, and columns without a pending scale cost
+// one read of the scale.
 __global__ void __launch_bounds__(GL_THREADS) k_gl_apply_scale(float* g, int64_t n, int R, const float* scale,
                                                                const int32_t* vgid, uint32_t* signs, int sign_words)
 {
     const int lane = threadIdx.x & 31, nb = (R + 31) / 32;
-    const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32);
-    for (int64_t x = ((int64_t)blockIdx.x * GL_THREADS + threadIdx.x) >> 5; x < n * nb; x += warps) {
-        const int64_t v = x / nb;
-        const int blk = (int)(x - v * nb), r = 32 * blk + lane;
-        const float sc = r < R ? scale[(vgid ? (int64_t)vgid[v] : 0) * R + r] : 1.0f;
-        if (!__any_sync(0xffffffffu, sc != 1.0f)) continue;
-        float y = 0.f;
-        if (r < R) {
-            y = g[v * R + r] * sc;
-            g[v * R + r] = y;
+    const int64_t warps = (int64_t)gridDim.x * (GL_THREADS / 32), quads = sb_cdiv(n, 4);
+    for (int64_t x = ((int64_t)blockIdx.x * GL_THREADS + threadIdx.x) >> 5; x < quads * nb; x += warps) {
+        const int64_t q = x / nb;
+        const int blk = (int)(x - q * nb), r = 32 * blk + lane;
+        float sc[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int64_t v = 4 * q + i;
+            sc[i] = 1.0f;
+            if (r < R && v < n) sc[i] = scale[(vgid ? (int64_t)vgid[v] : 0) * R + r];
         }
-        if (signs) {
-            const uint32_t w = sign_word(r < R && is_neg(y), R % 4 == 0);
-            if (lane == 0) signs[v * sign_words + blk] = w;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int64_t v = 4 * q + i;
+            if (!__any_sync(0xffffffffu, sc[i] != 1.0f)) continue;
+            float y = 0.f;
+            if (r < R) {
+                y = g[v * R + r] * sc[i];
+                g[v * R + r] = y;
+            }
+            if (signs) {
+                const uint32_t w = sign_word(r < R && is_neg(y), R % 4 == 0);
+                if (lane == 0) signs[v * sign_words + blk] = w;
+            }
         }
     }
 }
@@ -732,24 +761,16 @@ __global__ void __launch_bounds__(GL_THREADS) k_gl_fwd_graph(const int2* __restr
     }
 }
 
-__global__ void k_gl_copy_F(const uint32_t* counts, int64_t GR, int R, int64_t KS, int32_t* out)
-{
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < GR; r += (int64_t)gridDim.x * blockDim.x)
-        out[r] = (int32_t)counts[r / R * KS + sign_slot((int)(r % R), R % 4 == 0)];
-}
-
 // ----------------------------------------------------------------- host
-// sign words per vertex (32-bit, even) and frustration counters per graph
+// sign words per vertex (32-bit, even)
 static int gl_sign_words(int R) { return 2 * (int)sb_cdiv(R, 64); }
-static int64_t gl_slots(int R) { return 64 * sb_cdiv(R, 64); }
 
 static sb_status gl_scratch(sb_ctx* c, int R)
 {
     SB_TRY(sb_ensure(c, (void**)&c->gl_partial, &c->gl_partial_cap,
                      sizeof(float) * (size_t)std::max<int64_t>(c->n_gl_partials, 1) * R));
     SB_TRY(sb_ensure(c, (void**)&c->gl_red, &c->gl_red_cap, sizeof(double) * (size_t)c->num_sms * 8 * R));
-    const int64_t G = c->batch_G > 0 ? c->batch_G : 1;
-    return sb_ensure(c, (void**)&c->gl_misc, &c->gl_misc_cap, sizeof(int32_t) * (size_t)(G * gl_slots(R)));
+    return sb_ensure(c, (void**)&c->gl_misc, &c->gl_misc_cap, sizeof(int32_t) * (size_t)R);
 }
 
 static sb_status gl_signs_scratch(sb_ctx* c, int R, int copies)
@@ -758,12 +779,13 @@ static sb_status gl_signs_scratch(sb_ctx* c, int R, int copies)
                      sizeof(uint32_t) * (size_t)c->n * gl_sign_words(R) * copies);
 }
 
-static sb_status gl_signs_launch(sb_ctx* c, const float* gamma, int R, uint32_t* signs)
+// (clear: nclear counters set to zero, nullable)
+static sb_status gl_signs_launch(sb_ctx* c, const float* gamma, int R, uint32_t* signs, int32_t* clear, int64_t nclear)
 {
     const int sw = gl_sign_words(R);
     const unsigned blocks =
-        (unsigned)std::min<int64_t>(sb_cdiv(c->n * sw, GL_THREADS / 32), (int64_t)c->num_sms * 8);
-    k_gl_signs<<<blocks, GL_THREADS, 0, c->stream>>>(gamma, c->n, R, signs, sw);
+        (unsigned)std::min<int64_t>(sb_cdiv(c->n * sw, 8 * (GL_THREADS / 32)), (int64_t)c->num_sms * 8);
+    k_gl_signs<<<blocks, GL_THREADS, 0, c->stream>>>(gamma, c->n, R, signs, sw, clear, nclear);
     return sb_after_launch(c, "k_gl_signs");
 }
 
@@ -777,8 +799,8 @@ static const void* gl_count_kernel(int W)
                    : (const void*)k_gl_count<1>;
 }
 
-// adds the frustrated edges of every column to `counts` (gl_slots per graph)
-static sb_status gl_count_launch(sb_ctx* c, const uint32_t* signs, int R, uint32_t* counts)
+// adds the frustrated edges of every (graph, column) to F
+static sb_status gl_count_launch(sb_ctx* c, const uint32_t* signs, int R, int32_t* F)
 {
     if (c->m == 0) return SB_OK;
     int W = gl_sign_words(R) / 2;
@@ -788,13 +810,13 @@ static sb_status gl_count_launch(sb_ctx* c, const uint32_t* signs, int R, uint32
         // a warp takes at least 64 edges
         const unsigned bx = (unsigned)std::max<int64_t>(
             1, std::min<int64_t>(sb_cdiv(m, 64 * (GL_THREADS / 32)), sb_cdiv((int64_t)c->num_sms * 8, std::min(W, 8))));
-        k_gl_count_graphs<<<dim3(bx, (unsigned)W), GL_THREADS, 0, c->stream>>>(edges, m, c->vgid, (const uint64_t*)signs, W, gl_slots(R), counts);
+        k_gl_count_graphs<<<dim3(bx, (unsigned)W), GL_THREADS, 0, c->stream>>>(edges, m, c->vgid, (const uint64_t*)signs, W, R, F);
         return sb_after_launch(c, "k_gl_count_graphs");
     }
     // a warp takes at least 4 batches of 8 edges per group
     const int64_t batches = sb_cdiv(m * std::min(W, 32), 8 * 32 * 4 * (GL_THREADS / 32));
     const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(batches, (int64_t)c->num_sms * 4));
-    void* args[] = {(void*)&edges, &m, (void*)&signs, &W, &counts};
+    void* args[] = {(void*)&edges, &m, (void*)&signs, &W, &R, &F};
     SB_CHECK_CUDA(c, cudaLaunchKernel(gl_count_kernel(W), dim3(bx, (unsigned)sb_cdiv(W, 32)), dim3(GL_THREADS), args, 0, c->stream));
     return sb_after_launch(c, "k_gl_count");
 }
@@ -939,31 +961,22 @@ extern "C" sb_status sb_graphL_bwd(sb_ctx* c, const float* gamma, int32_t R, con
     return gl_rows_launch<false>(c, A);
 }
 
-// discrete loss of every (graph, column) from the sign words
-static sb_status gl_count_F(sb_ctx* c, const uint32_t* signs, int R, int32_t* F_out)
-{
-    const int64_t G = c->batch_G > 0 ? c->batch_G : 1, KS = gl_slots(R), GR = G * R;
-    uint32_t* counts = (uint32_t*)c->gl_misc;
-    SB_CHECK_CUDA(c, cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)(G * KS), c->stream));
-    SB_TRY(gl_count_launch(c, signs, R, counts));
-    k_gl_copy_F<<<(unsigned)std::min<int64_t>(sb_cdiv(GR, 256), (int64_t)c->num_sms * 16), 256, 0, c->stream>>>(
-        counts, GR, R, KS, F_out);
-    return sb_after_launch(c, "k_gl_copy_F");
-}
-
 extern "C" sb_status sb_graphL_round(sb_ctx* c, const float* gamma, int32_t R, int32_t* F_out, uint64_t* flip_out)
 {
     SB_TRY(gl_check(c, R));
     if (!gamma || !F_out) return sb_fail(c, SB_ERR_ARG, "null pointer");
-    SB_TRY(gl_scratch(c, R));
     SB_TRY(gl_signs_scratch(c, R, 1));
     SbProf prof(c, SB_PROF_GL_FWD);
-    SB_TRY(gl_signs_launch(c, gamma, R, c->gl_signs));
-    SB_TRY(gl_count_F(c, c->gl_signs, R, F_out));
-    if (flip_out && c->m > 0) {
-        const int64_t units = sb_cdiv(sb_cdiv(c->m, 64), 4) * sb_cdiv(R, 32);
-        k_gl_flips<<<(unsigned)std::min<int64_t>(sb_cdiv(units, GL_THREADS / 32), (int64_t)c->num_sms * 8), GL_THREADS, 0,
-                     c->stream>>>(c->edges, c->m, c->gl_signs, gl_sign_words(R), R, flip_out);
+    // two launches, three for the flips of a batch: 2.5 us each is what counts on
+    // a small graph
+    SB_TRY(gl_signs_launch(c, gamma, R, c->gl_signs, F_out, (c->batch_G > 0 ? c->batch_G : 1) * (int64_t)R));
+    const bool flips = flip_out && c->m > 0;
+    if (!flips || c->batch_G > 0) SB_TRY(gl_count_launch(c, c->gl_signs, R, F_out));
+    if (flips) {
+        const int64_t nb = sb_cdiv(R, 32), units = sb_cdiv(sb_cdiv(c->m, 64), 4) * nb;
+        const int64_t blocks = std::min<int64_t>(sb_cdiv(units, GL_THREADS / 32), (int64_t)c->num_sms * 8);
+        k_gl_flips<<<(unsigned)(sb_cdiv(blocks, nb) * nb), GL_THREADS, 0, c->stream>>>(
+            c->edges, c->m, c->gl_signs, gl_sign_words(R), R, flip_out, c->batch_G > 0 ? nullptr : F_out);
         return sb_after_launch(c, "k_gl_flips");
     }
     return SB_OK;
@@ -985,19 +998,16 @@ static sb_status gl_descent_graph(sb_ctx* c, GlArgs& A, const uint64_t* key, con
         c->capturing = true;
         sb_status st = SB_OK;
         const float* cur = src;
-        uint32_t* counts = (uint32_t*)c->gl_misc;
         for (int s = 0; s < steps && st == SB_OK; s++) {
             A.gin = cur;
             A.gout_rows = dst[s & 1];
             // sign words of step s's input: buffer s & 1
             A.signs = F_trace && s + 1 < steps ? c->gl_signs + ((s + 1) & 1) * sign_len : nullptr;
             if (s == steps - 1) A.signs = sign_last;
-            if (F_trace) st = gl_count_launch(c, c->gl_signs + (s & 1) * sign_len, A.R, counts);
+            if (F_trace) st = gl_count_launch(c, c->gl_signs + (s & 1) * sign_len, A.R, F_trace + (int64_t)s * GR);
             if (st == SB_OK) st = gl_rows_launch<true>(c, A);
             if (st == SB_OK) {
-                k_gl_step_final<<<rb, 256, 0, c->stream>>>(GR, A.R, gl_slots(A.R), c->gl_colmax, counts,
-                                                           F_trace ? F_trace + (int64_t)s * GR : nullptr, c->gl_scale,
-                                                           exps_out, renorm_log2);
+                k_gl_step_final<<<rb, 256, 0, c->stream>>>(GR, c->gl_colmax, c->gl_scale, exps_out, renorm_log2);
                 st = sb_after_launch(c, "k_gl_step_final");
             }
             cur = A.gout_rows;
@@ -1046,7 +1056,8 @@ extern "C" sb_status sb_graphL_descent(sb_ctx* c, const float* gamma0, float* ga
         SB_TRY(gl_signs_scratch(c, R, F_trace ? 2 : 1));
         SB_CHECK_CUDA(c, cudaMemsetAsync(c->gl_signs, 0, sizeof(uint32_t) * (size_t)c->n * sw * (F_trace ? 2 : 1), c->stream));
     }
-    SB_CHECK_CUDA(c, cudaMemsetAsync(c->gl_misc, 0, sizeof(int32_t) * (size_t)(GR / R * gl_slots(R)), c->stream));
+    if (F_trace && steps > 0) SB_CHECK_CUDA(c, cudaMemsetAsync(F_trace, 0, sizeof(int32_t) * (size_t)GR * steps, c->stream));
+    if (F_final) SB_CHECK_CUDA(c, cudaMemsetAsync(F_final, 0, sizeof(int32_t) * (size_t)GR, c->stream));
     SB_CHECK_CUDA(c, cudaMemsetAsync(c->gl_colmax, 0, sizeof(uint32_t) * GR, c->stream));
     SB_CHECK_CUDA(c, cudaMemsetAsync(exps_out, 0, sizeof(int32_t) * GR, c->stream));
     unsigned rb = (unsigned)sb_cdiv(GR, 256);
@@ -1061,7 +1072,7 @@ extern "C" sb_status sb_graphL_descent(sb_ctx* c, const float* gamma0, float* ga
         SB_CHECK_CUDA(c, cudaMemcpyAsync(c->gl_buf, gamma0, bytes, cudaMemcpyDeviceToDevice, c->stream));
         src = c->gl_buf;
     }
-    if (F_trace && steps > 0) SB_TRY(gl_signs_launch(c, src, R, c->gl_signs));
+    if (F_trace && steps > 0) SB_TRY(gl_signs_launch(c, src, R, c->gl_signs, nullptr, 0));
     uint32_t* const sign_last = !F_final ? nullptr : c->gl_signs + (F_trace ? (size_t)(steps & 1) * c->n * sw : 0);
     GlArgs A = gl_args(c, R);
     A.scale = c->gl_scale;
@@ -1100,7 +1111,7 @@ extern "C" sb_status sb_graphL_descent(sb_ctx* c, const float* gamma0, float* ga
     }
     // pending power-of-two scale of the last step
     if (steps > 0) {
-        const unsigned gb = (unsigned)std::min<int64_t>(sb_cdiv(c->n * sb_cdiv(R, 32), GL_THREADS / 32),
+        const unsigned gb = (unsigned)std::min<int64_t>(sb_cdiv(sb_cdiv(c->n, 4) * sb_cdiv(R, 32), GL_THREADS / 32),
                                                         (int64_t)c->num_sms * 8);
         k_gl_apply_scale<<<gb, GL_THREADS, 0, c->stream>>>(gamma_out, c->n, R, c->gl_scale,
                                                            c->batch_G > 0 ? c->vgid : nullptr, sign_last, sw);
@@ -1108,8 +1119,8 @@ extern "C" sb_status sb_graphL_descent(sb_ctx* c, const float* gamma0, float* ga
     }
     if (F_final) {
         SbProf prof(c, SB_PROF_GL_FWD);
-        if (steps == 0) SB_TRY(gl_signs_launch(c, gamma_out, R, sign_last));
-        SB_TRY(gl_count_F(c, sign_last, R, F_final));
+        if (steps == 0) SB_TRY(gl_signs_launch(c, gamma_out, R, sign_last, nullptr, 0));
+        SB_TRY(gl_count_launch(c, sign_last, R, F_final));
     }
     return SB_OK;
 }

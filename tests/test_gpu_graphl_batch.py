@@ -55,6 +55,27 @@ def test_batch_losses_flips_and_trace_match_oracle(loaded, R):
     assert np.array_equal(last.cpu().numpy().reshape(G, R), _round(refs, off, out.cpu().numpy())[0])
 
 
+@pytest.mark.parametrize("R", [5, 100])
+def test_rounding_takes_few_launches(loaded, R):
+    """On a small graph the launches are what a rounding costs: two, and one more
+    for the flips of a batch."""
+    import paper_2311_00869_gb300 as P
+
+    def launches(sb, flip):
+        gam = torch.rand((sb.n, R), device="cuda") * 2 - 1
+        sb.profile_read()
+        sb.graphL_round(gam, want_flip=flip)
+        return sum(k for _, k in sb.profile_read().values())
+
+    sb = P.SignedBal(0)
+    try:
+        sb.load_graph(*synth.random_connected(300, 800, 0.3, seed=3))
+        assert launches(sb, False) <= 2 and launches(sb, True) <= 2
+    finally:
+        sb.close()
+    assert launches(loaded[0], False) <= 2 and launches(loaded[0], True) <= 3
+
+
 def _ms(fn, reps=5):
     best = np.inf
     for _ in range(reps + 1):
