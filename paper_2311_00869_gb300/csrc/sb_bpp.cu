@@ -42,9 +42,18 @@
 // here 13.9 / 506 (30 per cent one by one 14.2 / 523, everything 14.7 / 570: a
 // ticket is an atomic on one counter).  Narrower groups: BFS_FIXED_PCT per cent
 // in advance, the rest 4 per group and ticket (39.2 ms on 512 uneven graphs,
-// 43.2 all in advance).
+// 43.2 all in advance).  A launch of fewer rounds than BFS_TICKET_ROUNDS (whole
+// warps) or BFS_TICKET_ROUNDS_NARROW deals everything out: there every warp draws
+// a ticket at each level for hardly any work.  Uniform random graph of 100,000
+// vertices and degree 10, one and 64 trees (1.5 rounds): 262 / 397 us with
+// tickets, 126 / 184 without; grid of 300 x 300 (352 and 565 levels) 8.3 / 18.6
+// against 4.0 / 7.8 ms.  Whole warps, R-MAT: 23,000 vertices (5 rounds), 250 trees
+// 507 with tickets, 544 without; 85,000 (20 rounds), 500 trees 1.28 / 1.50 ms.
+// Narrow: 100,000 vertices, 500 trees (12 rounds) 704 / 747 us.
 #define BFS_SINGLE_PCT 10
 #define BFS_FIXED_PCT 40
+#define BFS_TICKET_ROUNDS 4
+#define BFS_TICKET_ROUNDS_NARROW 8
 #define BFS_THREADS 128
 #define BFS_THREADS_PAR 128
 // Candidate-queue entries per lane (more are hashed lane by lane).
@@ -937,7 +946,8 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
     A.ls = ls;
     {
         const int64_t units = c->n_items * slices, groups = (int64_t)nblocks * (BD / G), rounds = units / groups;
-        A.fixed_rounds = G == 32 ? 1 : std::max<int64_t>(1, rounds * BFS_FIXED_PCT / 100);
+        const bool tickets = rounds >= (G == 32 ? BFS_TICKET_ROUNDS : BFS_TICKET_ROUNDS_NARROW);
+        A.fixed_rounds = !tickets ? sb_cdiv(units, groups) : G == 32 ? 1 : std::max<int64_t>(1, rounds * BFS_FIXED_PCT / 100);
         A.single_tickets = G == 32 ? units * BFS_SINGLE_PCT / 100 : 0;
         A.grab = G == 32 && rounds >= 1000 ? 8 : 4;
     }
