@@ -69,11 +69,16 @@
 #define BFS_ORDER_MIN (1 << 18)
 // Threads per SM below which a launch spreads its half-words over more lanes.
 #define BFS_SPREAD_THREADS 512
-// Work items below which a graph of mean degree 16 and more does so too, up to
-// 32 lanes per vertex.  Fewest lanes against 32, 128 / 500 trees: 15,000
-// vertices of degree 27 0.77 / 0.98 against 0.57 / 0.68 ms, 95,000 of degree 22
-// 1.24 / 1.35 against 0.91 / 1.20; 180,000 of degree 23 1.19 / 1.87 against
-// 1.57 / 2.06; 100,000 of degree 10 0.60 / 0.83 against 0.83 / 1.04.
+// Work items below which a graph of mean degree 16 and more with split rows does
+// so too, up to 32 lanes per vertex.  Fewest lanes against 32, R-MAT, 1 / 64 /
+// 250 trees: 14,000 vertices of degree 66 215 / 567 / 741 against 146 / 346 / 421
+// us, 23,000 of degree 30 198 / 516 / 843 against 149 / 417 / 544, 85,000 of degree
+// 34 450 / 970 / 995 against 433 / 789 / 1020; 180,000 of degree 23 (128 / 500
+// trees) 1.19 / 1.87 against 1.57 / 2.06 ms.  Where degrees are alike (no split
+// row) the vertices of a warp do not wait for one another, and few lanes are
+// faster: uniform random graphs, 30,000 vertices of degree 60 112 / 169 / 300
+// against 199 / 401 / 555 us, 100,000 of degree 60 185 / 311 / 927 against 510 /
+// 1341 / 1666.
 #define BFS_SPREAD_ITEMS (1 << 17)
 #define SYNC_WORDS 48
 // Shared-memory slots: rows of one owner thread's 32 trees (running minima,
@@ -899,9 +904,9 @@ static sb_status run_bfs(sb_ctx* c, int w0, int Wb, int32_t* parents)
         G = Gt;
         ls = 1;
     }
-    // and so does a dense one that fills them a few times over only: its rows
-    // take long, and whole warps hash without a queue
-    const bool dense = c->n_items < BFS_SPREAD_ITEMS && 2 * c->m >= 16 * c->n;
+    // and so does a dense one of uneven degrees that fills them a few times over
+    // only: its rows take long, and whole warps hash without a queue
+    const bool dense = c->n_items < BFS_SPREAD_ITEMS && 2 * c->m >= 16 * c->n && c->n_hubs > 0;
     while (!asked && G < 32 && (dense || c->n_items * slices * G < (int64_t)c->num_sms * BFS_SPREAD_THREADS)) {
         G <<= 1;
         ls++;
