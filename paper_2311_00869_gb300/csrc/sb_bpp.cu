@@ -187,6 +187,25 @@ __device__ __forceinline__ int group_excl_scan(int x, unsigned gmask, int gl, in
     return incl - x;
 }
 
+// Sum and maximum over the lanes of a group narrower than a warp.  By shuffles: a
+// warp-wide reduction whose mask is a group's runs once per group of the warp
+// (500,000 vertices of degree 10: 526 against 452 us for one tree, 804 / 681 for
+// 64 trees in 16 groups per warp).
+template <int G>
+__device__ __forceinline__ unsigned group_sum(unsigned x, unsigned gmask)
+{
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) x += __shfl_xor_sync(gmask, x, d);
+    return x;
+}
+template <int G>
+__device__ __forceinline__ unsigned group_max(unsigned x, unsigned gmask)
+{
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) x = max(x, __shfl_xor_sync(gmask, x, d));
+    return x;
+}
+
 // Hashes one lane's candidates m of neighbour u (label word lw), two at a time
 // (the highest and the lowest: the same one when a single candidate is left,
 // whose second update then repeats the first).
@@ -305,10 +324,10 @@ __device__ __forceinline__ void scan_row(const int32_t* cp, int len, const uint3
             once |= f[k];
             cnt += __popc(f[k]);
         }
-        const unsigned Tsum = __reduce_add_sync(gmask, (unsigned)cnt);
+        const unsigned Tsum = group_sum<G>((unsigned)cnt, gmask);
         if (Tsum == 0) continue;  // same for the whole group
         nhash += (uint32_t)cnt;
-        const unsigned cmax = __reduce_max_sync(gmask, (unsigned)cnt);
+        const unsigned cmax = group_max<G>((unsigned)cnt, gmask);
         if (cmax * G <= 4 * Tsum + 2 * G || Tsum > BFS_QUEUE * G) {
             // the lanes' shares are even enough (or too many to queue): every
             // lane hashes its own candidates into its own slots, two at a
