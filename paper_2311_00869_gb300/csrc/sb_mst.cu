@@ -64,6 +64,10 @@
 // 0.54 ms with light rounds, 0.40 without).
 #define MST_LIGHT_PAIRS (1ll << 26)
 #define MST_ROUNDS_MAX 64
+// Fewest vertices per graph for one component to sit out: finding it samples 32
+// edge ends per (graph, tree) and round, as many as a graph of 32 vertices has
+// rows (20,000 graphs of 9 vertices, 64 trees: 2.47 ms with, 1.34 without).
+#define MST_BIG_VERTICES 32
 
 struct MstArgs {
     int64_t n;
@@ -80,7 +84,7 @@ struct MstArgs {
     const int32_t* vgoff;  // first vertex of each vertex's graph (batches), or null
     const int32_t* voff;   // first vertex of each graph (batches), or null
     int64_t graphs;
-    uint32_t* big;         // [graph][tree]: root of the component that sits the round out
+    uint32_t* big;         // [graph][tree]: root of the component that sits the round out, or null
     uint32_t* P;
     uint32_t* R;
     uint64_t* B;
@@ -170,7 +174,7 @@ __global__ void __launch_bounds__(MST_THREADS) k_mst_big(MstArgs A, int r)
 {
     const int mode = mst_mode(A, r);
     if (blockIdx.x == 0 && threadIdx.x == 0) A.mode[r] = mode;
-    if (mode == MST_DONE || r == 0) return;
+    if (mode == MST_DONE || r == 0 || !A.big) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (MST_THREADS / 32);
     for (int64_t x = ((int64_t)blockIdx.x * MST_THREADS + threadIdx.x) >> 5; x < A.graphs * A.T; x += warps) {
@@ -221,7 +225,7 @@ __global__ void __launch_bounds__(MST_THREADS) k_mst_min(MstArgs A, int r)
         const int32_t v = q.x;
         const uint32_t c = ROUND0 ? (uint32_t)v : A.R[(int64_t)v * A.T + tt] >> 1;
         bool act = !((done >> lane) & 1u);
-        if (!ROUND0) act = act && c != A.big[(A.vgid ? (int64_t)A.vgid[v] * A.T : 0) + tt];
+        if (!ROUND0 && A.big) act = act && c != A.big[(A.vgid ? (int64_t)A.vgid[v] * A.T : 0) + tt];
         if (!__any_sync(0xffffffffu, act)) continue;
         const uint64_t kt = sb_tree_key(A.S, A.tree0 + A.tb0 + tt);
         const uint32_t base = A.vgoff ? (uint32_t)A.vgoff[v] : 0u;
@@ -285,7 +289,8 @@ __global__ void __launch_bounds__(MST_THREADS) k_mst_light(MstArgs A, int r)
         const int4 q = __ldg((const int4*)(A.items + item));
         const int32_t v = q.x;
         const uint32_t c = A.R[(int64_t)v * A.T + tt] >> 1;
-        const bool act = !((done >> lane) & 1u) && c != A.big[(A.vgid ? (int64_t)A.vgid[v] * A.T : 0) + tt];
+        bool act = !((done >> lane) & 1u);
+        if (A.big) act = act && c != A.big[(A.vgid ? (int64_t)A.vgid[v] * A.T : 0) + tt];
         if (!__any_sync(0xffffffffu, act)) continue;
         const uint64_t kt = sb_tree_key(A.S, A.tree0 + A.tb0 + tt);
         const uint32_t base = A.vgoff ? (uint32_t)A.vgoff[v] : 0u;
@@ -522,7 +527,7 @@ extern "C" sb_status sb_sample_trees_kruskal(sb_ctx* c, uint64_t seed, int64_t t
     A.vgoff = c->batch_G > 0 ? c->vgoff : nullptr;
     A.voff = c->batch_G > 0 ? c->b_voff : nullptr;
     A.graphs = graphs;
-    A.big = c->mst_big;
+    A.big = n >= MST_BIG_VERTICES * graphs ? c->mst_big : nullptr;
     A.P = c->mst_P;
     A.R = c->mst_R;
     A.B = c->mst_B;
@@ -540,7 +545,7 @@ extern "C" sb_status sb_sample_trees_kruskal(sb_ctx* c, uint64_t seed, int64_t t
     const unsigned grid_min =
         (unsigned)std::min<int64_t>(sb_cdiv(c->n_gl_items * T, MST_THREADS), (int64_t)c->num_sms * 16);
     const unsigned grid_big =
-        (unsigned)std::min<int64_t>(sb_cdiv(graphs * T * 32, MST_THREADS), (int64_t)c->num_sms * 16);
+        A.big ? (unsigned)std::min<int64_t>(sb_cdiv(graphs * T * 32, MST_THREADS), (int64_t)c->num_sms * 16) : 1u;
     SbProf prof(c, SB_PROF_BFS);
     for (int w0 = 0; w0 < W; w0 += Wp) {
         A.tb0 = 64 * (int64_t)w0;
