@@ -495,14 +495,15 @@ NCU_TRAFFIC = {
 
 
 def bfs_shape(sb):
-    """(words per BFS launch, lanes per vertex group) the library will use."""
+    """(words per BFS launch, lanes per vertex group) the library will use on a
+    graph that fills the GPU: a lane per half-word, up to a warp, or two when
+    the knob asks for them."""
     t = sb.get_tuning()
     words = t["bfs_words"] or 32
-    gw = 1
-    while gw < words:
-        gw <<= 1
-    g = t["bfs_group"]
-    return words, (g if gw < g <= 2 * gw else gw)
+    lanes = 2
+    while lanes < 2 * words and lanes < 32:
+        lanes <<= 1
+    return words, (2 * lanes if t["bfs_group"] == 2 * lanes else lanes)
 
 
 def traffic_bytes(fam, workload, shape):
