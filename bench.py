@@ -400,7 +400,7 @@ def main():
         "vs_baseline": None, "dtype": "u64", "data": "synthetic", "config": config_dict(args, n1, m1, world),
         "gpu_launches": launches, "clocks": r["clk"], "stages_ms_per_step": stages(prof, args.steps),
     }
-    line["roofline"] = roofline(prof, n1, m1, K, r["stats"], peak_hps, workload_name(args), bfs_shape(sb))
+    line["roofline"] = roofline(prof, n1, m1, K, r["stats"], peak_hps, workload_name(args), bfs_shape(sb, K))
     extras["roofline_score"] = roofline_family("score", prof, n1, m1, K)
     extras["roofline_hash"] = roofline_family("hash", prof, n1, m1, K)
     if not args.no_extras and rank == 0:
@@ -450,7 +450,7 @@ def side_legs(P, args, stream, peak_hps, K=1024, steps=10, warmup=3):
                "edge_evals_per_s": K * m1 / (r["ms_step"] / 1000.0), "trees_per_s": K / (r["ms_step"] / 1000.0),
                "stages_ms_per_step": stages(r["prof"], steps), "bfs_stats": r["stats"], "tuning": tuned,
                "roofline": roofline_family("bfs", r["prof"], n1, m1, K, r["stats"], peak_hps,
-                                           traffic_bytes("bfs", WORKLOAD_NAMES["rmat20"], bfs_shape(sb))),
+                                           traffic_bytes("bfs", WORKLOAD_NAMES["rmat20"], bfs_shape(sb, K))),
                "roofline_score": roofline_family("score", r["prof"], n1, m1, K),
                "fr_min": int(r["fr_min"])}
         out["plain_vs_batched"] = plain_leg(sb, m1)
@@ -494,12 +494,12 @@ NCU_TRAFFIC = {
 }
 
 
-def bfs_shape(sb):
-    """(words per BFS launch, lanes per vertex group) the library will use on a
-    graph that fills the GPU: a lane per half-word, up to a warp, or two when
-    the knob asks for them."""
+def bfs_shape(sb, K):
+    """(words per BFS launch, lanes per vertex group) the library will use for K
+    trees on a graph that fills the GPU: a lane per half-word, up to a warp, or
+    two when the knob asks for them."""
     t = sb.get_tuning()
-    words = t["bfs_words"] or 32
+    words = min(t["bfs_words"] or 32, (K + 63) // 64)
     lanes = 2
     while lanes < 2 * words and lanes < 32:
         lanes <<= 1

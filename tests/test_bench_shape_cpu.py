@@ -16,11 +16,12 @@ class _Tuned:
         return self.knobs
 
 
-@pytest.mark.parametrize("words,group,want", [(0, 0, (32, 32)), (32, 32, (32, 32)), (16, 0, (16, 32)), (16, 16, (16, 32)),
-                                              (8, 0, (8, 16)), (8, 32, (8, 32)), (8, 8, (8, 16)), (4, 32, (4, 8)),
-                                              (1, 0, (1, 2)), (1, 4, (1, 4)), (5, 0, (5, 16))])
-def test_bfs_shape_follows_the_library(words, group, want):
+@pytest.mark.parametrize("words,group,K,want", [
+    (0, 0, 4096, (32, 32)), (32, 32, 4096, (32, 32)), (16, 0, 4096, (16, 32)), (16, 16, 4096, (16, 32)),
+    (0, 0, 1024, (16, 32)), (32, 0, 1024, (16, 32)), (8, 0, 1024, (8, 16)), (8, 32, 1024, (8, 32)), (8, 8, 1024, (8, 16)),
+    (4, 32, 1024, (4, 8)), (0, 0, 1, (1, 2)), (1, 4, 4096, (1, 4)), (0, 0, 300, (5, 16))])
+def test_bfs_shape_follows_the_library(words, group, K, want):
     spec = importlib.util.spec_from_file_location("bench_shape_under_test", os.path.join(ROOT, "bench.py"))
     bench = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(bench)
-    assert bench.bfs_shape(_Tuned(words, group)) == want
+    assert bench.bfs_shape(_Tuned(words, group), K) == want
