@@ -1226,8 +1226,12 @@ static sb_status bfs_enqueue(sb_ctx* c, int32_t* parents_out)
         // 17 to 23 words leave most lanes of the second slice idle: 16 words
         // and the rest apart take less (1100 trees on the 2^20 R-MAT graph 18.6
         // against 26.4 ms; 1536, 24 words, 27.0 against 28.2, but 2.9 against
-        // 2.7 on 95,000 vertices)
-        if (Wb > 16 && Wb < 24) Wb = 16;
+        // 2.7 on 95,000 vertices).  Not so a graph of less than one round of
+        // whole warps, whose levels take the same time however many words they
+        // carry: 1100 trees, 1000 vertices 92 us in two launches, 57 in one, 3200
+        // (R-MAT) 592 / 397, a path of 2000 22.0 / 16.7 ms; 10,000 vertices 276
+        // / 329 us.
+        if (Wb > 16 && Wb < 24 && c->n_items * 32 >= (int64_t)c->num_sms * BFS_BLOCKS_PER_SM * BFS_THREADS) Wb = 16;
         SB_TRY(run_bfs(c, w0, Wb, parents_out));
     }
     return SB_OK;

@@ -81,15 +81,16 @@ def test_dealt_out_and_by_tickets(P, n, K):
         sb.close()
 
 
-@pytest.mark.parametrize("K", [1030, 1100, 1472])  # 17, 18 and 23 words
-def test_words_split_over_two_launches(P, K):
-    n, u, v, s = _hub_graph(1500, 2600, 700, seed=64)
+# 17, 18 and 23 words: two launches, one on a graph too small to fill a round
+@pytest.mark.parametrize("n,K,launches", [(6000, 1030, 2), (6000, 1100, 2), (6000, 1472, 2), (1500, 1030, 1), (1500, 1472, 1)])
+def test_words_split_over_two_launches(P, n, K, launches):
+    n, u, v, s = _hub_graph(n, 2 * n, 700, seed=64)
     g = O.clean_graph(n, u, v, s)
     sb = P.SignedBal(0)
     try:
         sb.load_graph(n, u, v, s)
         par = sb.sample_trees(9, 3, K, want_parents=True)
-        assert sb.stats()["bfs_launches"] == 2
+        assert sb.stats()["bfs_launches"] == launches
         counts, hashes = sb.frustration()
         ref = O.sample(g, 9, 3, K, want_labels=True, want_parents=True)
         assert np.array_equal(counts.cpu().numpy(), ref["counts"])
