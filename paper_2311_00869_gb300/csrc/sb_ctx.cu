@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t* __res
 // starts then put the tile in order in shared memory, and the writes go out as
 // runs of equal digits (128 bytes on average).  16.8 M keys: 126 us a pass, 158
 // when three barriers ended every round of 256 keys; 3 or 5 blocks per SM 145,
-// 155 us.
+// 155 us (4 leave 64 registers, at which 84 bytes per thread spill).
 __global__ void __launch_bounds__(RS_THREADS, RS_BLOCKS) k_radix_scatter(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                                                               int64_t n, int shift, unsigned mask,
                                                               const int32_t* __restrict__ ofs, int64_t ntiles)

@@ -17,7 +17,10 @@
 // Blocks per SM the row kernel's registers must allow, and neighbour rows loaded
 // before they are added.  Descent step on the 2^20 R-MAT graph, 256 columns:
 // 3.12 / 2.92 / 2.94 ms at 4 / 5 / 6 blocks and 4 rows, 2.98 at 8 blocks and 2
-// rows, 3.66 / 3.64 at 3 / 4 blocks and 8 rows (spills).
+// rows, 3.66 / 3.64 at 3 / 4 blocks and 8 rows.  The 5 blocks leave 48 registers,
+// at which the step kernels spill 200 to 260 bytes per thread and the gradient's
+// 50 to 90 (the four-piece strided step 100 to 170 at 64 registers); that costs
+// less than the warps that more registers would take.
 #define GL_ROWS_MIN_BLOCKS 5
 #define GL_INFLIGHT 4
 

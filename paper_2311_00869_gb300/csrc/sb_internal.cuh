@@ -176,7 +176,8 @@ struct sb_ctx {
     sb_cloud_slot* cl_table = nullptr;
     sb_cloud_entry* cl_entries = nullptr;
     uint64_t* cl_bits = nullptr;   // [ceil(n/64)][cl_max] state bits, chunk-major
-    int32_t* cl_meta = nullptr;    // [0] n_states, [1] overflow, [2] mismatches
+    int32_t* cl_meta = nullptr;    // [0] n_states, [1] overflow, [2] 1 when a tree of the batch needs the exact
+                                   // comparison again (which ones: cl_mismatch)
     int32_t* cl_assign = nullptr;  // K: state per tree of the batch
     int32_t* cl_rep = nullptr;     // cl_max: batch tree that created the state in this batch, else -1
     int32_t* cl_mismatch = nullptr;// K
